@@ -124,6 +124,53 @@ def test_sampler_matches_inverse_cdf(T, vocab):
     assert flags <= 1
 
 
+@pytest.mark.parametrize("rows,vocab,offset", [
+    (1, 1, 0), (3, 127, 1), (2, 2048, 3), (5, 2049, 0), (1, 8191, 2), (152, 8192, 0), (1, 16384, 0),
+    (77, 16385, 0), (1, 32000, 0), (500, 8001, 1), (200, 32003, 1), (2, 65537, 0), (3, 131071, 0), (2, 131072, 3),
+])
+def test_sampler_slices(rows, vocab, offset):
+    """Vocabularies at the edges of a 128-id tile, a CTA's slice and the largest
+    cluster, rows whose first logit is not 16-byte aligned (offset floats past an
+    aligned address, odd vocabularies), few and many rows: the drawn id is the
+    inverse CDF's, or u lies within fp32 rounding of the boundary (bound 1e-5: the
+    sums are of at most 131072 terms in a tree, relative error below 40 * 2^-24)."""
+    from paper_2608_10362_gb300 import op_sample
+    z = gen_logits(21, rows, vocab, scale=2.0)
+    z[0, vocab - 1] = 12.0               # mass at the end of the last slice
+    u = ((2 * np.random.default_rng(6).integers(0, 1 << 23, rows) + 1) * 2.0 ** -24).astype(np.float32)
+    u[rows - 1] = 1 - 2.0 ** -24
+    buf = torch.empty(rows * vocab + offset, dtype=torch.float32, device="cuda")
+    zt = buf[offset:].view(rows, vocab)
+    zt.copy_(torch.from_numpy(z))
+    for T in (0.0, 0.9):
+        out = op_sample(zt, T, torch.from_numpy(u).cuda()).cpu().numpy()
+        for r in list(range(min(rows, 12))) + [rows - 1]:
+            expect = draft_token(z[r].astype(np.float64), T, float(u[r]))
+            if out[r] != expect:
+                c = np.cumsum(softmax_t(z[r], T))
+                assert T > 0 and abs(u[r] - c[min(out[r], expect)]) < 1e-5, (r, T, out[r], expect)
+
+
+def test_sampler_degenerate_rows():
+    """Rows without a proper distribution: a NaN among the logits, +inf, every
+    logit -inf but one, all equal; the draw is an id of the row (the first argmax
+    where the weights have no finite sum)."""
+    from paper_2608_10362_gb300 import op_sample
+    V = 32000
+    z = gen_logits(22, 5, V, scale=1.0)
+    z[0, 17000] = np.nan
+    z[1, 29000] = np.inf
+    z[2, :] = -np.inf
+    z[2, 31999] = -3.0
+    z[3, :] = 0.0
+    u = np.full(5, 0.5, dtype=np.float32)
+    out = op_sample(torch.from_numpy(z).cuda(), 1.0, torch.from_numpy(u).cuda()).cpu().numpy()
+    assert out[0] == int(np.nanargmax(z[0])) and out[1] == 29000 and out[2] == 31999
+    assert abs(int(out[3]) - V // 2) <= 1
+    g = op_sample(torch.from_numpy(z).cuda(), 0.0).cpu().numpy()
+    assert g[0] == int(np.nanargmax(z[0])) and g[1] == 29000 and g[2] == 31999 and g[3] == 0
+
+
 @pytest.fixture(scope="module")
 def tiny_engine():
     from paper_2608_10362_gb300 import Engine
