@@ -64,6 +64,20 @@ bool encode_map(CUtensorMap* map, const void* base, int rows, int cols, int box_
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Packed tiles (16 KB each, contiguous) as rows of 256 bf16, box {256, 32}: one tile
+// per box, copied as stored.
+bool encode_packed(CUtensorMap* map, const void* base, long long tiles) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (fn == nullptr || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
+  cuuint64_t dims[2] = {256, static_cast<cuuint64_t>(tiles) * 32};
+  cuuint64_t strides[1] = {512};
+  cuuint32_t box[2] = {256, 32};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // 3-D bf16 tensor map, no swizzle (the bytes are copied as stored), zero fill
 // out of bounds: dims {d0, d1, d2} elements, strides of dims 1 and 2 in bytes,
 // box {b0, b1, b2}.
@@ -103,6 +117,11 @@ bool ensure_func_attrs() {
   cudaError_t e = gemm_set_max_smem();
   if (e != cudaSuccess) {
     g_attr_error = std::string("gemm smem attribute: ") + cudaGetErrorString(e);
+    return false;
+  }
+  e = gemm_pair_set_max_smem();
+  if (e != cudaSuccess) {
+    g_attr_error = std::string("pair gemm smem attribute: ") + cudaGetErrorString(e);
     return false;
   }
   e = attention_set_max_smem();
@@ -452,7 +471,11 @@ size_t layout_workspace(const memspec_init_params* p, memspec_ctx* c, uint8_t* b
   const size_t o_ol = w.take(static_cast<size_t>(kMaxRows) * qmax_dim * 2);
   const size_t o_act = w.take(static_cast<size_t>(kMaxRows) * fmax * 2);
   const size_t o_actl = w.take(static_cast<size_t>(kMaxRows) * fmax * 2);
-  const size_t o_gp = w.take(static_cast<size_t>(2) * nsm * kMaxRows * 128 * 4);
+  // split-K partials: two slots per CTA, or (gemm_pair.cu, every projection but the
+  // LM head) one per row tile and one more per CTA
+  const int proj_rt = std::max({ceil_div(fmax, 64), ceil_div(model_q(t) + 2 * model_kv(t), 128),
+                                has_draft ? ceil_div(model_q(dm) + 2 * model_kv(dm), 128) : 1, ceil_div(dmax, 128)});
+  const size_t o_gp = w.take(static_cast<size_t>(std::max(2 * nsm, proj_rt + 1 + nsm)) * kMaxRows * 128 * 4);
   const size_t o_gc = w.take(static_cast<size_t>(max_rt) * 4);   // split-K arrival counters
   const size_t o_apo = w.take(po * 4);
   const size_t o_apml = w.take(po / 64 * 2 * 4 + 1024);
@@ -722,8 +745,42 @@ CskPick pick_csk(const GemmArgs& a, int planes, int g0) {
   return best;
 }
 
-void emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) {
+// CTA pairs of gemm_pair.cu for `rows` activation rows, 0: gemm.cu's kernel.  One
+// pair per two SMs, and ranges of at least a quarter of a row-tile pair.
+// Two planes: from 17 rows.  Verify pass of 6 layers of the 8B target, this kernel /
+// gemm.cu's: 18 rows 0.784 / 0.836 ms, 54 rows 0.911 / 1.060, 144 rows 1.292 / 1.559.
+// One plane (memspec_op_linear): from 161 rows.  28672 x 4096 at 144 rows 57.1 / 58.2
+// us but 12288 x 4096 27.2 / 25.9; at 256 rows 71.5 / 85.6 and 32.3 / 35.0.
+int gemm_pairs(int rows, int split, int row_tiles, int k_tiles) {
+  if (rows < (split ? 17 : 161)) return 0;
+  const int T = (row_tiles + 1) / 2 * k_tiles;
+  return std::max(1, std::min(sm_count() / 2, T / std::max(1, (k_tiles + 3) / 4)));
+}
+
+memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) {
   const int planes = a.split ? 2 : 1;
+  a.partials = c->gemm_part;
+  a.counters = c->gemm_cnt;
+  a.status = c->status;
+  a.pairs = c->pass_kernel ? 0 : gemm_pairs(a.rows_total, a.split, a.row_tiles, a.k_tiles);
+  if (a.pairs > 0) {
+    if (a.a_packed != nullptr &&
+        !encode_packed(&a.map_a, a.a_packed, static_cast<long long>(a.row_tiles) * a.k_tiles))
+      return fail(c, MEMSPEC_ERR_CUDA, "weight tensor map");
+    a.warm = 0;
+    a.csk = 0;
+    a.stages = gemm_pair_stages(a.n_pad, a.split, a.epi);
+    PassOp op{};
+    op.type = OP_GEMM;
+    op.grid = a.pairs;
+    op.u.g = a;
+    ops.push_back(op);
+    if (a.epi != EPI_F32 || !sk_split_free((a.row_tiles + 1) / 2 * a.k_tiles, a.k_tiles, a.pairs)) {
+      op.type = OP_GEMM_EPI;
+      ops.push_back(op);
+    }
+    return MEMSPEC_OK;
+  }
   if (a.warm < 0) a.warm = warm_down();   // the down projection marks itself with -1
   else a.warm = warm_other();
   int grid = gemm_grid(a.row_tiles, a.k_tiles);
@@ -734,9 +791,6 @@ void emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) {
     a.csk = pk.csk;
   }
   a.stages = gemm_pick_stages(a.n_pad, planes, a.csk);
-  a.partials = c->gemm_part;
-  a.counters = c->gemm_cnt;
-  a.status = c->status;
   // Two or more 16-row chunks (trees, batched verify, prefill): split row tiles
   // get their own epilogue launch, one CTA per (row tile, 16-row chunk), instead
   // of one contributor folding every chunk in turn (a 31-node tree step 5.02 ->
@@ -760,6 +814,7 @@ void emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) {
     ep.u.g = a;
     ops.push_back(ep);
   }
+  return MEMSPEC_OK;
 }
 
 // Launches as separate kernels: the op after the embedding kernel (which writes
@@ -772,7 +827,7 @@ void mark_ctx_early(std::vector<PassOp>& ops, size_t first) {
   if (!enabled || ops.size() < first + 2 || ops[first].type != OP_EMBED) return;
   ops[first + 1].full_dep = 1;
   for (size_t i = first + 2; i < ops.size(); ++i) {
-    if (ops[i].type == OP_GEMM) ops[i].u.g.ctx_early = 1;
+    if (ops[i].type == OP_GEMM || ops[i].type == OP_GEMM_EPI) ops[i].u.g.ctx_early = 1;
     if (ops[i].type == OP_ATTN) ops[i].u.at.ctx_early = 1;
   }
 }
@@ -783,7 +838,10 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
   const memspec_model_cfg& cf = m.cfg;
   const int d = cf.d_model, qd = model_q(cf), kvd = model_kv(cf), F = cf.d_ffn;
   const int rows = f.n_groups * f.R;
-  const int n_pad = round_up(rows, 16);
+  // the pair kernel pads the rows and reads the activations in boxes of its own
+  const bool pair_rows = !c->pass_kernel && gemm_pairs(rows, 1, 1, 1) > 0;
+  const int n_pad = pair_rows ? gemm_pair_pad(rows, 1) : round_up(rows, 16);
+  const int box = pair_rows ? gemm_pair_box_rows(n_pad, 1) : n_pad;
   const int hsel = cf.head_dim == 128 ? 1 : 0;
   EmbedArgs ea{};
   ea.mode = f.mode;
@@ -838,8 +896,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(a.n_out, 128);
       a.k_tiles = ceil_div(d, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->xg, rows, d, n_pad, &a.map_b) ||
-          !act_map(c, c->xg_lo, rows, d, n_pad, &a.map_b2))
+      if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
+          !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.rms = 1;
@@ -859,7 +917,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.rope_cos = c->rope_cos[hsel];
       a.rope_sin = c->rope_sin[hsel];
       a.plan = c->plan;
-      emit_gemm(c, a, ops);
+      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
     }
     {  // attention
       AttnArgs at{};
@@ -908,8 +966,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(d, 128);
       a.k_tiles = ceil_div(qd, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->o, rows, qd, n_pad, &a.map_b) ||
-          !act_map(c, c->o_lo, rows, qd, n_pad, &a.map_b2))
+      if (!act_map(c, c->o, rows, qd, box, &a.map_b) ||
+          !act_map(c, c->o_lo, rows, qd, box, &a.map_b2))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.epi = EPI_RESIDUAL;
@@ -921,7 +979,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.xg_lo_out = c->xg_lo;
       a.ss_stride = c->ss_stride;
       a.plan = c->plan;
-      emit_gemm(c, a, ops);
+      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
       ss_count = ceil_div(d, 128);
     }
     {  // gate/up + SwiGLU
@@ -935,8 +993,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(F, 64);
       a.k_tiles = ceil_div(d, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->xg, rows, d, n_pad, &a.map_b) ||
-          !act_map(c, c->xg_lo, rows, d, n_pad, &a.map_b2))
+      if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
+          !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.rms = 1;
@@ -949,7 +1007,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.act_lo = c->act_lo;
       a.act_ld = F;
       a.plan = c->plan;
-      emit_gemm(c, a, ops);
+      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
     }
     {  // down projection + residual
       GemmArgs a{};
@@ -962,8 +1020,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(d, 128);
       a.k_tiles = ceil_div(F, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->act, rows, F, n_pad, &a.map_b) ||
-          !act_map(c, c->act_lo, rows, F, n_pad, &a.map_b2))
+      if (!act_map(c, c->act, rows, F, box, &a.map_b) ||
+          !act_map(c, c->act_lo, rows, F, box, &a.map_b2))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.epi = EPI_RESIDUAL;
@@ -976,7 +1034,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.xg_lo_out = c->xg_lo;
       a.ss_stride = c->ss_stride;
       a.plan = c->plan;
-      emit_gemm(c, a, ops);
+      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
     }
   }
   if (f.logits != nullptr) {  // final RMSNorm + LM head -> fp32 logits
@@ -992,8 +1050,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
     a.row_tiles = ceil_div(cf.vocab, 128);
     a.k_tiles = ceil_div(d, 64);
     a.l2_hint = m.l2_hint;
-    if (!act_map(c, c->xg, rows, d, n_pad, &a.map_b) ||
-        !act_map(c, c->xg_lo, rows, d, n_pad, &a.map_b2))
+    if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
+        !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
       return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
     a.split = 1;
     a.rms = 1;
@@ -1007,7 +1065,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
     a.last_only = f.last_only;
     a.out_group_stride = f.out_group_stride;
     a.plan = c->plan;
-    emit_gemm(c, a, ops);
+    if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
   }
   if (!c->pass_kernel) mark_ctx_early(ops, first_op);
   return MEMSPEC_OK;
@@ -1020,7 +1078,10 @@ memspec_status run_ops_separately(memspec_ctx* c, const std::vector<PassOp>& ops
     cudaError_t e = cudaSuccess;
     switch (op.type) {
       case OP_EMBED: e = launch_embed(op.u.e, op.n_units, c->main, c->pdl); break;
-      case OP_GEMM: e = launch_gemm(op.u.g, op.grid, op.smem, c->main, c->pdl && !op.full_dep); break;
+      case OP_GEMM:
+        e = op.u.g.pairs ? launch_gemm_pair(op.u.g, c->main, c->pdl && !op.full_dep)
+                         : launch_gemm(op.u.g, op.grid, op.smem, c->main, c->pdl && !op.full_dep);
+        break;
       case OP_GEMM_EPI: e = launch_gemm_split_epi(op.u.g, op.grid, c->main, c->pdl); break;
       case OP_ATTN: e = launch_attention(op.u.at, op.grid, c->main, c->pdl && !op.full_dep); break;
       case OP_SAMPLE: e = launch_sample(op.u.s, c->main, c->pdl); break;
@@ -2187,12 +2248,13 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
   a.n_out = n_out;
   a.k_in = k;
   a.rows_total = rows;
-  a.n_pad = n_pad;
   a.row_tiles = ceil_div(n_out, 128);
   a.k_tiles = ceil_div(k, 64);
-  a.stages = gemm_pick_stages(n_pad);
+  a.pairs = gemm_pairs(rows, 0, a.row_tiles, a.k_tiles);
+  a.n_pad = a.pairs ? gemm_pair_pad(rows, 0) : n_pad;
+  a.stages = a.pairs ? gemm_pair_stages(a.n_pad, 0, EPI_F32) : gemm_pick_stages(n_pad);
   a.l2_hint = L2_EVICT_FIRST;
-  if (!encode_map(&a.map_b, x, rows, k, n_pad)) {
+  if (!encode_map(&a.map_b, x, rows, k, a.pairs ? gemm_pair_box_rows(a.n_pad, 0) : n_pad)) {
     g_op_error = "cuTensorMapEncodeTiled failed for x";
     return MEMSPEC_ERR_CUDA;
   }
@@ -2207,14 +2269,16 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
                                : reinterpret_cast<uint32_t*>(sb + part_bytes +
                                                              align256(static_cast<size_t>(a.row_tiles) * 4));
   a.plan = nullptr;
-  const int grid = gemm_grid(a.row_tiles, a.k_tiles);
+  const int grid = a.pairs ? a.pairs : gemm_grid(a.row_tiles, a.k_tiles);
   // more than 16 rows: split row tiles finished by the split epilogue kernel (as
-  // in the passes)
-  a.split_epi = (n_pad >= 32 && !sk_split_free(a.row_tiles * a.k_tiles, a.k_tiles, grid)) ? 1 : 0;
-  cudaError_t e = launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages),
-                              static_cast<cudaStream_t>(stream), false);
+  // in the passes), which starts while the GEMM drains and waits for its end
+  const int units = a.pairs ? (a.row_tiles + 1) / 2 : a.row_tiles;
+  a.split_epi = (n_pad >= 32 && !sk_split_free(units * a.k_tiles, a.k_tiles, grid)) ? 1 : 0;
+  cudaError_t e = a.pairs ? launch_gemm_pair(a, static_cast<cudaStream_t>(stream), false)
+                          : launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages),
+                                        static_cast<cudaStream_t>(stream), false);
   if (e == cudaSuccess && a.split_epi)
-    e = launch_gemm_split_epi(a, grid, static_cast<cudaStream_t>(stream), false);
+    e = launch_gemm_split_epi(a, grid, static_cast<cudaStream_t>(stream), true);
   if (e != cudaSuccess) {
     g_op_error = std::string("gemm launch: ") + cudaGetErrorString(e);
     return MEMSPEC_ERR_CUDA;

@@ -347,52 +347,49 @@ __device__ __forceinline__ void rms_prologue(const GemmArgs& a, float* rms, int 
   named_bar_sync(1, 128);
 }
 
-// rms_prologue for the 16 rows of one chunk only (threads et < 16, the same
-// summation order, every partial sum of a row in flight at once); ends with a
-// barrier over the 128 threads.
-__device__ __forceinline__ void rms_chunk(const GemmArgs& a, float* rms, int chunk, int et) {
-  const int r = chunk * 16 + et;
-  if (et < 16 && r < a.n_pad) {
-    float val = 0.f;
-    if (r < a.rows_total) {
-      float sum = 0.f;
-      for (int i0 = 0; i0 < a.ss_count; i0 += 32) {
-        float t[32];
-#pragma unroll
-        for (int q = 0; q < 32; ++q)
-          t[q] = (i0 + q < a.ss_count) ? a.ss[static_cast<size_t>(i0 + q) * a.ss_stride + r] : 0.f;
-#pragma unroll
-        for (int q = 0; q < 32; ++q) sum += t[q];
-      }
-      val = rsqrtf(sum / static_cast<float>(a.k_in) + a.eps);
-    }
-    rms[r] = val;
-  }
-  named_bar_sync(1, 128);
+// Partial slot of row tile 2 unit + rank in CTA pair c (gemm_pair.cu), `sl` 0: the
+// first tile of its range, 1: the last.  The fp32-output epilogue leaves only split
+// tiles: two slots per CTA.  The others leave every tile: segments numbered along
+// the stream-K order, each of which starts a new unit or a new pair.
+__device__ __forceinline__ int pair_slot(const GemmArgs& a, int unit, int c, int rank, int sl) {
+  return a.epi == EPI_F32 ? 2 * (2 * c + rank) + sl : 2 * (unit + c) + rank;
+}
+
+// Split-K partials of slot `slot` (gemm.cu: 2 CTA + (0: the CTA's first row tile, 1:
+// its last)): [chunk of 16 rows][4 rows each][feature][4], so that a warp's 16-byte
+// stores and loads are contiguous.  Offset in floats of rows 0..3 of a chunk for
+// feature et; rows 4 q .. 4 q + 3 are q * 512 further.
+__device__ __forceinline__ size_t part_offset(int slot, int chunks, int chunk, int et) {
+  return (static_cast<size_t>(slot) * chunks + chunk) * (kTileM * 16) + et * 4;
 }
 
 // Sum of the split-K partials of row tile rt, chunk `chunk`, for feature et:
-// contributors in ascending CTA order, four fetched at once.
+// contributors in ascending CTA order, N fetched at once.  a.pairs (gemm_pair.cu):
+// rt is one of a pair of row tiles; contributors are CTA pairs, whose CTA rt % 2
+// holds this row tile.
+template <int N = 4>
 __device__ __forceinline__ void reduce_partials(const GemmArgs& a, int rt, int c_first, int c_last,
                                                 int chunk, int et, int T, int G, float* v) {
   const int KT = a.k_tiles;
+  const int chunks = (a.rows_total + 15) / 16;
+  const int unit = a.pairs ? rt >> 1 : rt;       // tile of the stream-K order
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = 0.f;
-  for (int cc0 = c_first; cc0 <= c_last; cc0 += 4) {
-    float4 tmp[4][4];
+  for (int cc0 = c_first; cc0 <= c_last; cc0 += N) {
+    float4 tmp[N][4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < N; ++q) {
       const int cc = cc0 + q;
       if (cc <= c_last) {
-        const int sl = (sk_begin(cc, T, G) >= rt * KT) ? 0 : 1;
-        const float* pp = a.partials + static_cast<size_t>(2 * cc + sl) * a.n_pad * kTileM +
-                          (static_cast<size_t>(chunk) * kTileM + et) * 16;
+        const int sl = (sk_begin(cc, T, G) >= unit * KT) ? 0 : 1;
+        const int slot = a.pairs ? pair_slot(a, unit, cc, rt & 1, sl) : 2 * cc + sl;
+        const float* pp = a.partials + part_offset(slot, chunks, chunk, et);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) tmp[q][e] = ld_cg_f4(pp + 4 * e);
+        for (int e = 0; e < 4; ++e) tmp[q][e] = ld_cg_f4(pp + e * kTileM * 4);
       }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < N; ++q) {
       if (cc0 + q <= c_last) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -541,17 +538,13 @@ __device__ __forceinline__ void epilogue_segment(const GemmArgs& a, const EpiCtx
         st_async_f4(raddr + 16 * q, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3], rbar);
     }
   } else {
-    // partial sums, chunk-major: the 16 rows of chunk k for feature et at
-    // ((k * 128) + et) * 16 (a warp's stores, and a reader's loads, of one chunk
-    // are one contiguous 2 KB run)
-    const int slot = (seg == 0) ? 0 : 1;
-    float* pb = a.partials + static_cast<size_t>(2 * c + slot) * a.n_pad * kTileM +
-                static_cast<size_t>(et) * 16;
     for (int chunk = 0; chunk < a.n_pad / 16; ++chunk) {
       load_chunk(chunk);
-      float4* dst = reinterpret_cast<float4*>(pb + static_cast<size_t>(chunk) * kTileM * 16);
+      float* dst = a.partials + part_offset(2 * c + (seg == 0 ? 0 : 1), a.n_pad / 16, chunk, et);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(dst + q * kTileM * 4) =
+            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
   }
   tc_fence_before();

@@ -137,11 +137,13 @@ struct GemmArgs {
   int ss_count, ss_stride;
   float eps;
   // split-K scratch
-  float* partials;          // [2 * grid][n_pad * 128]
+  float* partials;          // gemm.cu: [2 * grid][n_pad * 128]; gemm_pair.cu: pair_slot
   int* counters;            // [row_tiles], zero on entry, left zero
   int split_epi;            // 1: contributors to a split row tile only store their partials;
                             // gemm_split_epi_kernel (the next launch) sums them and runs the
                             // epilogue, one CTA per (row tile, 16-row chunk)
+  int pairs;                // > 0: gemm_pair.cu's kernel with this many CTA pairs (n_pad a
+                            // = gemm_pair_pad, map_b boxes of gemm_pair_box_rows rows)
   int csk;                  // > 1: launched in clusters of csk CTAs (n_pad == 16 only); a
                             // row tile whose contributors share a cluster is summed by
                             // its first contributor from partials the others push into
@@ -343,6 +345,13 @@ int gemm_pick_stages(int n_pad, int planes = 1, int csk = 0);
 int gemm_max_active_clusters(int epi, int csk, size_t smem);
 cudaError_t gemm_set_max_smem();
 cudaError_t launch_gemm_split_epi(const GemmArgs& a, int gemm_grid, cudaStream_t s, bool pdl);
+// gemm_pair.cu (stages, activation box rows and launch for n_pad rows in one plane
+// or, split, two)
+int gemm_pair_stages(int n_pad, int split, int epi);
+int gemm_pair_pad(int rows, int split);
+int gemm_pair_box_rows(int n_pad, int split);
+cudaError_t gemm_pair_set_max_smem();
+cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_attention(const AttnArgs& a, int n_groups, cudaStream_t s, bool pdl);
 size_t attention_smem_bytes(const AttnArgs& a);
 cudaError_t attention_set_max_smem();

@@ -4,6 +4,7 @@ and T = 1, a batch of four requests, the greedy stream against greedy
 target-only decoding, and prompt edge cases."""
 import numpy as np
 import pytest
+import torch
 
 from lockstep import LOGIT_TOL, RECORDS, LockstepReport, check_step
 from oracle.llama import LlamaOracle
@@ -152,3 +153,41 @@ def test_tiny_prompt_edge_cases(tiny):
         rep.record(f"tiny prompt length {n}")
         assert rep.steps == 4
         assert rep.band_flags == 0
+
+
+@pytest.mark.parametrize("B,K", [(2, 8), (3, 10), (8, 15), (9, 14), (10, 15), (16, 15)])
+def test_verify_pass_row_counts(B, K):
+    """One verify pass at 18, 33, 128, 135, 160 and 256 rows (the CTA-pair GEMM's
+    operand layouts: two planes side by side up to 128 rows, one after the other
+    above), requests of different lengths: every request's logits and new K/V against
+    the oracle at the step tests' tolerance."""
+    from oracle.llama import LlamaOracle
+    from paper_2608_10362_gb300 import Engine, _lib
+    from seeded_inputs import SHAPES, gen_prompt, gen_weights
+    t = SHAPES["tiny_target"]
+    wt = gen_weights(t, 0)
+    oracle = LlamaOracle(t, wt, keep_f64=True)
+    eng = Engine(t, wt, max_batch=B, max_seq=96, max_k=K, max_drafts=0, use_graphs=False)
+    try:
+        prompts = [gen_prompt(40 + b, 3 + 5 * (b % 7), t.vocab) for b in range(B)]
+        for b, p in enumerate(prompts):
+            eng.prefill(b, p, seed=b)
+        x = np.stack([gen_prompt(80 + b, K, t.vocab) for b in range(B)]).astype(np.int32)
+        eng.set_batch(B)
+        eng.write_buffer(_lib.BUF_DRAFT_TOKENS, x)
+        eng.verify_step(K)
+        assert eng.sync() == 0
+        z = eng.target_logits(B, K)
+        kv = eng.kv.view(torch.bfloat16).view(t.n_layers, 2, B, t.n_kv_heads, 96, t.head_dim).float().cpu().numpy()
+        for b, p in enumerate(prompts):
+            cache = oracle.new_cache(96)
+            rows = np.concatenate([p, x[b]])
+            ref = oracle.forward(cache, rows)[-(K + 1):]
+            assert np.abs(z[b] - ref).max() <= 1e-3 * np.abs(ref).max()
+            n = len(rows)
+            k_ref = np.stack([np.asarray(cache.k[l])[:n] for l in range(t.n_layers)])   # [layer][pos][head][hd]
+            got = kv[:, 0, b, :, :n].transpose(0, 2, 1, 3)
+            # bf16 values: at most one rounding step apart
+            assert np.abs(got - k_ref).max() <= 2.0 ** -7 * np.abs(k_ref).max()
+    finally:
+        eng.close()
