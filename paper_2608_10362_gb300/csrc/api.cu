@@ -64,6 +64,24 @@ bool encode_map(CUtensorMap* map, const void* base, int rows, int cols, int box_
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Activations for gemm_small.cu: `planes` row-major [rows][k] bf16 planes, plane_bytes
+// apart, k whole 64-column tiles, as {64 columns, rows, planes, k tiles}; box {64,
+// box_rows, planes, box_kt}, 128-byte swizzle, rows past `rows` read as zero.
+bool encode_x4(CUtensorMap* map, const void* base, int rows, int k, int planes, long long plane_bytes, int box_rows,
+               int box_kt) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (fn == nullptr || (reinterpret_cast<uintptr_t>(base) & 15) != 0 || k % 64 != 0) return false;
+  cuuint64_t dims[4] = {64, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes),
+                        static_cast<cuuint64_t>(k / 64)};
+  cuuint64_t strides[3] = {static_cast<cuuint64_t>(k) * 2, static_cast<cuuint64_t>(plane_bytes), 128};
+  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(planes),
+                       static_cast<cuuint32_t>(box_kt)};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Packed tiles (16 KB each, contiguous) as rows of 256 bf16, box {256, 32}: one tile
 // per box, copied as stored.
 bool encode_packed(CUtensorMap* map, const void* base, long long tiles) {
@@ -122,6 +140,11 @@ bool ensure_func_attrs() {
   e = gemm_pair_set_max_smem();
   if (e != cudaSuccess) {
     g_attr_error = std::string("pair gemm smem attribute: ") + cudaGetErrorString(e);
+    return false;
+  }
+  e = gemm_small_set_max_smem();
+  if (e != cudaSuccess) {
+    g_attr_error = std::string("small gemm smem attribute: ") + cudaGetErrorString(e);
     return false;
   }
   e = attention_set_max_smem();
@@ -632,6 +655,22 @@ bool act_map(memspec_ctx* c, const void* ptr, int rows, int cols, int n_pad, CUt
   return true;
 }
 
+// The activation maps of a projection: for the kernel that a pass over `rows` rows
+// runs (`pass`, the persistent pass kernel: 2-D maps of n_pad rows).
+bool pass_x(memspec_ctx* c, GemmArgs& a, bool pass, const bf16* hi, const bf16* lo, int rows, int k, int n_pad) {
+  int box = n_pad;
+  if (!pass) {
+    const long long apart = reinterpret_cast<const uint8_t*>(lo) - reinterpret_cast<const uint8_t*>(hi);
+    if (rows <= kSmallRows && k % 64 == 0 && apart > 0) {
+      a.x4d = 1;
+      return encode_x4(&a.map_b, hi, rows, k, 2, apart, 8, 1) &&
+             encode_x4(&a.map_b2, hi, rows, k, 2, apart, 8, gemm_small_x_group());
+    }
+    box = rows <= kSmallRows ? 8 : gemm_pair_box_rows(n_pad, 1);
+  }
+  return act_map(c, hi, rows, k, box, &a.map_b) && act_map(c, lo, rows, k, box, &a.map_b2);
+}
+
 // ---------------------------------------------------------------- forward pass
 struct FwdSpec {
   int mode, n_groups, R, j;
@@ -668,26 +707,7 @@ int gemm_grid(int row_tiles, int k_tiles) {
   return std::max(1, std::min({T, sms, T / min_tiles}));
 }
 
-// Whether a GEMM launch dry-runs its tail before griddepcontrol.wait: worth it
-// when the launch starts early (while its predecessor's CTAs drain); the down
-// projection follows gate/up, whose CTAs nearly all reduce and leave late.
-// MEMSPEC_WARM_DOWN / MEMSPEC_WARM_OTHER = 0 or 1 override (measurement).
-int warm_default(const char* env, int dflt) {
-  const char* e = std::getenv(env);
-  return e != nullptr ? (e[0] == '1') : dflt;
-}
-int warm_down() {
-  static int v = -1;
-  if (v < 0) v = warm_default("MEMSPEC_WARM_DOWN", 1);
-  return v;
-}
-int warm_other() {
-  static int v = -1;
-  if (v < 0) v = warm_default("MEMSPEC_WARM_OTHER", 1);
-  return v;
-}
-
-// Cluster exchange for decode GEMMs (16 padded rows): a grid of Q clusters of C
+// Cluster exchange for decode GEMMs (gemm_small.cu): a grid of Q clusters of C
 // CTAs whose stream-K ranges put every split row tile inside one cluster, so that
 // the split-K partials move through distributed shared memory instead of global
 // memory (no store, counter or reload on the critical tail).  Taken when its
@@ -716,18 +736,17 @@ CskPick pick_csk(const GemmArgs& a, int planes, int g0) {
   static const int c_max = std::min(8, env_int("MEMSPEC_CSK_MAX", 4));
   const int R = a.row_tiles, KT = a.k_tiles, T = R * KT;
   CskPick best{g0, 0};
-  if (!enabled || a.n_pad != 16 || sk_split_free(T, KT, g0)) return best;
+  if (!enabled || sk_split_free(T, KT, g0)) return best;
   int best_cost = ceil_div(T, g0) + kCskTailTiles;
   int dev = 0;
   cudaGetDevice(&dev);
-  static std::map<std::tuple<int, int, int, size_t>, int> fit;   // (device, epi, C, smem) -> clusters
+  static std::map<std::tuple<int, int, int, int>, int> fit;   // (device, epi, planes, C) -> clusters
   static std::mutex fit_mu;
   std::lock_guard<std::mutex> lock(fit_mu);
   for (int C = 2; C <= c_max; ++C) {
-    const size_t smem = gemm_smem_bytes(a.n_pad, gemm_pick_stages(a.n_pad, planes, C), planes, C);
-    const auto key = std::make_tuple(dev, a.epi, C, smem);
+    const auto key = std::make_tuple(dev, a.epi, planes, C);
     auto it = fit.find(key);
-    if (it == fit.end()) it = fit.emplace(key, gemm_max_active_clusters(a.epi, C, smem)).first;
+    if (it == fit.end()) it = fit.emplace(key, gemm_small_max_clusters(a.epi, planes, C)).first;
     // never more CTAs than plain stream-K: clusters must all be resident while the
     // previous launch still holds SMs (a larger clustered grid measured far slower)
     const int q_max = std::min({it->second, g0 / C, T / C});
@@ -747,28 +766,38 @@ CskPick pick_csk(const GemmArgs& a, int planes, int g0) {
 
 // CTA pairs of gemm_pair.cu for `rows` activation rows, 0: gemm.cu's kernel.  One
 // pair per two SMs, and ranges of at least a quarter of a row-tile pair.
-// Two planes: from 17 rows.  Verify pass of 6 layers of the 8B target, this kernel /
+// Two planes: from 9 rows (gemm_small.cu takes up to 8).  Verify pass of 6 layers of the 8B target, this kernel /
 // gemm.cu's: 18 rows 0.784 / 0.836 ms, 54 rows 0.911 / 1.060, 144 rows 1.292 / 1.559.
 // One plane (memspec_op_linear): from 161 rows.  28672 x 4096 at 144 rows 57.1 / 58.2
 // us but 12288 x 4096 27.2 / 25.9; at 256 rows 71.5 / 85.6 and 32.3 / 35.0.
 int gemm_pairs(int rows, int split, int row_tiles, int k_tiles) {
-  if (rows < (split ? 17 : 161)) return 0;
+  if (rows < (split ? 9 : 161)) return 0;
   const int T = (row_tiles + 1) / 2 * k_tiles;
   return std::max(1, std::min(sm_count() / 2, T / std::max(1, (k_tiles + 3) / 4)));
 }
 
-memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) {
+// gemm_small.cu's launch of a projection: grid, cluster exchange, ring.
+void small_gemm(GemmArgs& a, int* grid) {
+  const int planes = a.split ? 2 : 1;
+  const CskPick pk = pick_csk(a, planes, gemm_grid(a.row_tiles, a.k_tiles));
+  *grid = pk.grid;
+  a.small = 1;
+  a.csk = pk.csk;
+  a.n_pad = 16;
+  a.stages = gemm_small_stages(planes, a.csk);
+}
+
+// `pass`: an op of the persistent pass kernel.
+memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, bool pass, std::vector<PassOp>& ops) {
   const int planes = a.split ? 2 : 1;
   a.partials = c->gemm_part;
   a.counters = c->gemm_cnt;
   a.status = c->status;
-  a.pairs = c->pass_kernel ? 0 : gemm_pairs(a.rows_total, a.split, a.row_tiles, a.k_tiles);
+  a.pairs = pass ? 0 : gemm_pairs(a.rows_total, a.split, a.row_tiles, a.k_tiles);
   if (a.pairs > 0) {
     if (a.a_packed != nullptr &&
         !encode_packed(&a.map_a, a.a_packed, static_cast<long long>(a.row_tiles) * a.k_tiles))
       return fail(c, MEMSPEC_ERR_CUDA, "weight tensor map");
-    a.warm = 0;
-    a.csk = 0;
     a.stages = gemm_pair_stages(a.n_pad, a.split, a.epi);
     PassOp op{};
     op.type = OP_GEMM;
@@ -781,39 +810,17 @@ memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, std::vector<PassOp>& ops) 
     }
     return MEMSPEC_OK;
   }
-  if (a.warm < 0) a.warm = warm_down();   // the down projection marks itself with -1
-  else a.warm = warm_other();
-  int grid = gemm_grid(a.row_tiles, a.k_tiles);
-  a.csk = 0;
-  if (!c->pass_kernel) {   // the persistent kernel runs every op on its own grid
-    const CskPick pk = pick_csk(a, planes, grid);
-    grid = pk.grid;
-    a.csk = pk.csk;
-  }
-  a.stages = gemm_pick_stages(a.n_pad, planes, a.csk);
-  // Two or more 16-row chunks (trees, batched verify, prefill): split row tiles
-  // get their own epilogue launch, one CTA per (row tile, 16-row chunk), instead
-  // of one contributor folding every chunk in turn (a 31-node tree step 5.02 ->
-  // 4.81 ms, batched 8B verify 17.6 -> 12.0 ms).  MEMSPEC_SPLIT_EPI_ROWS sets the
-  // threshold (0: never; measurement).
-  static const int split_rows = env_int("MEMSPEC_SPLIT_EPI_ROWS", 32);
-  a.split_epi = (!c->pass_kernel && a.csk == 0 && split_rows > 0 && a.n_pad >= split_rows &&
-                 !sk_split_free(a.row_tiles * a.k_tiles, a.k_tiles, grid))
-                    ? 1
-                    : 0;
   PassOp op{};
   op.type = OP_GEMM;
-  op.grid = grid;
-  op.smem = static_cast<int>(gemm_smem_bytes(a.n_pad, a.stages, planes, a.csk));
+  op.grid = gemm_grid(a.row_tiles, a.k_tiles);
+  if (pass) {   // the persistent kernel runs every op on its own grid
+    a.stages = gemm_pick_stages(a.n_pad, planes);
+    op.smem = static_cast<int>(gemm_smem_bytes(a.n_pad, a.stages, planes));
+  } else {
+    small_gemm(a, &op.grid);
+  }
   op.u.g = a;
   ops.push_back(op);
-  if (a.split_epi) {
-    PassOp ep{};
-    ep.type = OP_GEMM_EPI;
-    ep.grid = grid;
-    ep.u.g = a;
-    ops.push_back(ep);
-  }
   return MEMSPEC_OK;
 }
 
@@ -838,10 +845,9 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
   const memspec_model_cfg& cf = m.cfg;
   const int d = cf.d_model, qd = model_q(cf), kvd = model_kv(cf), F = cf.d_ffn;
   const int rows = f.n_groups * f.R;
-  // the pair kernel pads the rows and reads the activations in boxes of its own
-  const bool pair_rows = !c->pass_kernel && gemm_pairs(rows, 1, 1, 1) > 0;
-  const int n_pad = pair_rows ? gemm_pair_pad(rows, 1) : round_up(rows, 16);
-  const int box = pair_rows ? gemm_pair_box_rows(n_pad, 1) : n_pad;
+  // prefill chunks and tree passes are separate launches in every mode
+  const bool pass = c->pass_kernel && f.mode != PLAN_PREFILL && f.mode != PLAN_TREE;
+  const int n_pad = !pass && rows > kSmallRows ? gemm_pair_pad(rows, 1) : round_up(rows, 16);
   const int hsel = cf.head_dim == 128 ? 1 : 0;
   EmbedArgs ea{};
   ea.mode = f.mode;
@@ -896,8 +902,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(a.n_out, 128);
       a.k_tiles = ceil_div(d, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
-          !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
+      if (!pass_x(c, a, pass, c->xg, c->xg_lo, rows, d, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.rms = 1;
@@ -917,7 +922,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.rope_cos = c->rope_cos[hsel];
       a.rope_sin = c->rope_sin[hsel];
       a.plan = c->plan;
-      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
+      if (memspec_status s = emit_gemm(c, a, pass, ops); s != MEMSPEC_OK) return s;
     }
     {  // attention
       AttnArgs at{};
@@ -942,7 +947,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       at.plan = c->plan;
       at.status = c->status;
       // per-op launches stream K/V tiles by TMA (the persistent pass kernel keeps cp.async)
-      if (!c->pass_kernel) {
+      if (!pass) {
         const int kv_rows = c->p.max_batch * cf.n_kv_heads * c->p.max_seq;
         if (!encode_map(&at.kmap, kl, kv_rows, cf.head_dim, 64) ||
             !encode_map(&at.vmap, vl, kv_rows, cf.head_dim, 64))
@@ -966,8 +971,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(d, 128);
       a.k_tiles = ceil_div(qd, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->o, rows, qd, box, &a.map_b) ||
-          !act_map(c, c->o_lo, rows, qd, box, &a.map_b2))
+      if (!pass_x(c, a, pass, c->o, c->o_lo, rows, qd, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.epi = EPI_RESIDUAL;
@@ -979,7 +983,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.xg_lo_out = c->xg_lo;
       a.ss_stride = c->ss_stride;
       a.plan = c->plan;
-      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
+      if (memspec_status s = emit_gemm(c, a, pass, ops); s != MEMSPEC_OK) return s;
       ss_count = ceil_div(d, 128);
     }
     {  // gate/up + SwiGLU
@@ -993,8 +997,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(F, 64);
       a.k_tiles = ceil_div(d, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
-          !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
+      if (!pass_x(c, a, pass, c->xg, c->xg_lo, rows, d, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.rms = 1;
@@ -1007,11 +1010,10 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.act_lo = c->act_lo;
       a.act_ld = F;
       a.plan = c->plan;
-      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
+      if (memspec_status s = emit_gemm(c, a, pass, ops); s != MEMSPEC_OK) return s;
     }
     {  // down projection + residual
       GemmArgs a{};
-      a.warm = -1;
       a.a_packed = m.w + m.lay.wdown[l];
       a.n_out = d;
       a.k_in = F;
@@ -1020,8 +1022,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.row_tiles = ceil_div(d, 128);
       a.k_tiles = ceil_div(F, 64);
       a.l2_hint = m.l2_hint;
-      if (!act_map(c, c->act, rows, F, box, &a.map_b) ||
-          !act_map(c, c->act_lo, rows, F, box, &a.map_b2))
+      if (!pass_x(c, a, pass, c->act, c->act_lo, rows, F, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
       a.epi = EPI_RESIDUAL;
@@ -1034,7 +1035,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       a.xg_lo_out = c->xg_lo;
       a.ss_stride = c->ss_stride;
       a.plan = c->plan;
-      if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
+      if (memspec_status s = emit_gemm(c, a, pass, ops); s != MEMSPEC_OK) return s;
     }
   }
   if (f.logits != nullptr) {  // final RMSNorm + LM head -> fp32 logits
@@ -1050,8 +1051,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
     a.row_tiles = ceil_div(cf.vocab, 128);
     a.k_tiles = ceil_div(d, 64);
     a.l2_hint = m.l2_hint;
-    if (!act_map(c, c->xg, rows, d, box, &a.map_b) ||
-        !act_map(c, c->xg_lo, rows, d, box, &a.map_b2))
+    if (!pass_x(c, a, pass, c->xg, c->xg_lo, rows, d, n_pad))
       return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
     a.split = 1;
     a.rms = 1;
@@ -1065,9 +1065,9 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
     a.last_only = f.last_only;
     a.out_group_stride = f.out_group_stride;
     a.plan = c->plan;
-    if (memspec_status s = emit_gemm(c, a, ops); s != MEMSPEC_OK) return s;
+    if (memspec_status s = emit_gemm(c, a, pass, ops); s != MEMSPEC_OK) return s;
   }
-  if (!c->pass_kernel) mark_ctx_early(ops, first_op);
+  if (!pass) mark_ctx_early(ops, first_op);
   return MEMSPEC_OK;
 }
 
@@ -1080,7 +1080,7 @@ memspec_status run_ops_separately(memspec_ctx* c, const std::vector<PassOp>& ops
       case OP_EMBED: e = launch_embed(op.u.e, op.n_units, c->main, c->pdl); break;
       case OP_GEMM:
         e = op.u.g.pairs ? launch_gemm_pair(op.u.g, c->main, c->pdl && !op.full_dep)
-                         : launch_gemm(op.u.g, op.grid, op.smem, c->main, c->pdl && !op.full_dep);
+                         : launch_gemm_small(op.u.g, op.grid, c->main, c->pdl && !op.full_dep);
         break;
       case OP_GEMM_EPI: e = launch_gemm_split_epi(op.u.g, op.grid, c->main, c->pdl); break;
       case OP_ATTN: e = launch_attention(op.u.at, op.grid, c->main, c->pdl && !op.full_dep); break;
@@ -2250,14 +2250,7 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
   a.rows_total = rows;
   a.row_tiles = ceil_div(n_out, 128);
   a.k_tiles = ceil_div(k, 64);
-  a.pairs = gemm_pairs(rows, 0, a.row_tiles, a.k_tiles);
-  a.n_pad = a.pairs ? gemm_pair_pad(rows, 0) : n_pad;
-  a.stages = a.pairs ? gemm_pair_stages(a.n_pad, 0, EPI_F32) : gemm_pick_stages(n_pad);
   a.l2_hint = L2_EVICT_FIRST;
-  if (!encode_map(&a.map_b, x, rows, k, a.pairs ? gemm_pair_box_rows(a.n_pad, 0) : n_pad)) {
-    g_op_error = "cuTensorMapEncodeTiled failed for x";
-    return MEMSPEC_ERR_CUDA;
-  }
   a.epi = EPI_F32;
   a.out = y;
   a.out_ld = n_out;
@@ -2269,16 +2262,36 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
                                : reinterpret_cast<uint32_t*>(sb + part_bytes +
                                                              align256(static_cast<size_t>(a.row_tiles) * 4));
   a.plan = nullptr;
-  const int grid = a.pairs ? a.pairs : gemm_grid(a.row_tiles, a.k_tiles);
-  // more than 16 rows: split row tiles finished by the split epilogue kernel (as
-  // in the passes), which starts while the GEMM drains and waits for its end
-  const int units = a.pairs ? (a.row_tiles + 1) / 2 : a.row_tiles;
-  a.split_epi = (n_pad >= 32 && !sk_split_free(units * a.k_tiles, a.k_tiles, grid)) ? 1 : 0;
-  cudaError_t e = a.pairs ? launch_gemm_pair(a, static_cast<cudaStream_t>(stream), false)
-                          : launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages),
-                                        static_cast<cudaStream_t>(stream), false);
-  if (e == cudaSuccess && a.split_epi)
-    e = launch_gemm_split_epi(a, grid, static_cast<cudaStream_t>(stream), true);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  bool maps;
+  cudaError_t e = cudaSuccess;
+  if (rows <= 16) {   // gemm_small.cu, rows of one plane
+    int grid;
+    small_gemm(a, &grid);
+    a.x4d = k % 64 == 0 ? 1 : 0;
+    maps = a.x4d ? encode_x4(&a.map_b, x, rows, k, 1, static_cast<long long>(k) * 2, 16, 1) &&
+                       encode_x4(&a.map_b2, x, rows, k, 1, static_cast<long long>(k) * 2, 16, gemm_small_x_group())
+                 : encode_map(&a.map_b, x, rows, k, 16);
+    if (maps) e = launch_gemm_small(a, grid, st, false);
+  } else {
+    a.pairs = gemm_pairs(rows, 0, a.row_tiles, a.k_tiles);
+    a.n_pad = a.pairs ? gemm_pair_pad(rows, 0) : n_pad;
+    a.stages = a.pairs ? gemm_pair_stages(a.n_pad, 0, EPI_F32) : gemm_pick_stages(n_pad);
+    maps = encode_map(&a.map_b, x, rows, k, a.pairs ? gemm_pair_box_rows(a.n_pad, 0) : n_pad);
+    const int grid = a.pairs ? a.pairs : gemm_grid(a.row_tiles, a.k_tiles);
+    // split row tiles are finished by the next launch, which starts while the GEMM
+    // drains and waits for its end
+    const int units = a.pairs ? (a.row_tiles + 1) / 2 : a.row_tiles;
+    a.split_epi = sk_split_free(units * a.k_tiles, a.k_tiles, grid) ? 0 : 1;
+    if (maps)
+      e = a.pairs ? launch_gemm_pair(a, st, false)
+                  : launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages), st, false);
+    if (maps && e == cudaSuccess && a.split_epi) e = launch_gemm_split_epi(a, grid, st, true);
+  }
+  if (!maps) {
+    g_op_error = "cuTensorMapEncodeTiled failed for x";
+    return MEMSPEC_ERR_CUDA;
+  }
   if (e != cudaSuccess) {
     g_op_error = std::string("gemm launch: ") + cudaGetErrorString(e);
     return MEMSPEC_ERR_CUDA;

@@ -1,10 +1,10 @@
-// gemm.cu - weight-streaming projection GEMM for the verify and draft passes.
+// gemm.cu - weight-streaming projection GEMM with fp32 output (memspec_op_linear from
+// 17 to 160 rows, memspec_op_linear_noalloc); the persistent pass kernel streams its
+// projections the same way.
 //
-// Y[rows][n_out] = X[rows][k] . W[n_out][k]^T with rows <= 256 (K+1 verify rows,
-// 1-2 draft rows, up to 128 prefill rows).  At these row counts every projection
-// of the decoder (QKV, O, gate/up, down, LM head) reads each weight exactly once
-// and is bound by HBM bandwidth, so the kernel is organised around streaming
-// weights:
+// Y[rows][n_out] = X[rows][k] . W[n_out][k]^T with rows <= 256.  At these row counts
+// every projection reads each weight exactly once and is bound by HBM bandwidth, so
+// the kernel is organised around streaming weights:
 //
 //  * swap-AB: the weight tile is the MMA's M=128 operand, the activation rows
 //    are its N (16..256) operand; tcgen05.mma.kind::f16 (bf16 in, fp32 out)
@@ -22,9 +22,6 @@
 //    per CTA, one CTA per SM; a row tile split over several CTAs is reduced by
 //    the last-arriving CTA in ascending CTA order (deterministic, no float
 //    atomics) from an fp32 partial buffer;
-//  * fused epilogues: fp32 logits; residual add (+ the row sums of squares
-//    the next RMSNorm needs); SwiGLU of interleaved gate/up tiles; RoPE on q/k
-//    with K/V appended to the KV cache at each row's position.
 #include <cuda_bf16.h>
 
 #include <cstdlib>
@@ -52,13 +49,9 @@ struct SmemCtl {
   int reduce_flag;
   int wait_ok;
   float red[4][16];
-  uint64_t recv;        // cluster exchange: partials pushed by peers (one phase)
-  int recv_pending;     // this CTA expects pushed partials it has not yet consumed
 };
 
-// CSK: launched in clusters of a.csk CTAs with the cluster exchange of split row
-// tiles (epilogue_segment); the plain kernel carries none of that code.
-template <int EPI, bool CSK>
+template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_constant__ GemmArgs a) {
   __shared__ SmemCtl ctl;
   extern __shared__ uint8_t dsmem_raw[];
@@ -73,8 +66,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
   float* stage = reinterpret_cast<float*>(smem_b + static_cast<size_t>(S) * b_bytes);
   float* rms = stage + kStageFloats;
   EpiCtx* ectx = reinterpret_cast<EpiCtx*>(rms + kMaxRows);
-  float* recv = reinterpret_cast<float*>(
-      (reinterpret_cast<uintptr_t>(ectx + 1) + 15) & ~static_cast<uintptr_t>(15));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int T = a.row_tiles * a.k_tiles;
@@ -95,10 +86,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
       mbar_init(&ctl.acc_empty[b], 4);
     }
     mbar_init(&ctl.drain, 1);
-    if constexpr (CSK) {
-      mbar_init(&ctl.recv, 1);
-      ctl.recv_pending = 0;
-    }
     ctl.abort_flag = 0;
     ctl.reduce_flag = 0;
     fence_mbar_init();
@@ -111,9 +98,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // cluster exchange: the barriers above are initialised before any peer pushes
-  // (every thread arrives here; a thread waits before its first push)
-  if constexpr (CSK) cluster_arrive_release();
   pdl_launch_dependents();
   const uint32_t tmem_base = ctl.tmem_base;
   // optional trace (16 slots per CTA): 0 entry, 13 dependency released,
@@ -210,42 +194,38 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc_bf16_f32(kTileM, layout == kWide ? 2 * a.n_pad : a.n_pad);
-      // descriptors of stage 0; a stage's (and a k-step's) are offsets in the
-      // start-address field (address >> 4, 14 bits: shared memory < 256 KB)
-      const uint64_t adesc0 = make_smem_desc_sw128(smem_addr(smem_a));
-      const uint64_t bdesc0 = make_smem_desc_sw128(smem_addr(smem_b));
-      const uint32_t a_step = kABytes >> 4, b_step = static_cast<uint32_t>(b_bytes) >> 4;
-      const uint32_t p_step = static_cast<uint32_t>(plane_bytes) >> 4;
-      int s = 0, seg = 0;
-      uint32_t ph = 0;
-      bool ok = true, first = true;
-      for (int t = t_begin; t < t_end && ok; ++seg) {
-        const int rt = t / KT;
-        const int seg_end = min(t_end, (rt + 1) * KT);
-        const int buf = seg & 1;
-        if (seg >= 2 &&
-            !mbar_wait_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>((seg >> 1) - 1) & 1u,
-                               abort_flag, a.status)) {
-          ok = false;
-          break;
-        }
+    // The whole warp walks the tiles and one elected lane issues, so that descriptors
+    // and loop counters stay in uniform registers.
+    const bool lead = elect_one();
+    const uint32_t idesc = make_idesc_bf16_f32(kTileM, layout == kWide ? 2 * a.n_pad : a.n_pad);
+    // descriptors of stage 0; a stage's (and a k-step's) are offsets in the
+    // start-address field (address >> 4, 14 bits: shared memory < 256 KB)
+    const uint64_t adesc0 = make_smem_desc_sw128(smem_addr(smem_a));
+    const uint64_t bdesc0 = make_smem_desc_sw128(smem_addr(smem_b));
+    const uint32_t a_step = kABytes >> 4, b_step = static_cast<uint32_t>(b_bytes) >> 4;
+    const uint32_t p_step = static_cast<uint32_t>(plane_bytes) >> 4;
+    int s = 0, seg = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = t_begin; t < t_end && ok; ++seg) {
+      const int seg_end = min(t_end, (t / KT + 1) * KT);
+      const int buf = seg & 1;
+      if (seg >= 2) {
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>((seg >> 1) - 1) & 1u,
+                                                       abort_flag, a.status));
+        if (!ok) break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * acols);
+      for (int tt = t; tt < seg_end; ++tt) {
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.full[s], ph, abort_flag, a.status));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * acols);
-        for (int tt = t; tt < seg_end; ++tt) {
-          if (!mbar_wait_bounded(&ctl.full[s], ph, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          if (first) {
-            trace_at(trace, 3);
-            first = false;
-          }
-          tc_fence_after();
-          const uint64_t ad = adesc0 + static_cast<uint32_t>(s) * a_step;
-          const uint64_t bd = bdesc0 + static_cast<uint32_t>(s) * b_step;
-          const uint32_t acc0 = tt > t ? 1u : 0u;
+        const uint64_t ad = adesc0 + static_cast<uint32_t>(s) * a_step;
+        const uint64_t bd = bdesc0 + static_cast<uint32_t>(s) * b_step;
+        const uint32_t acc0 = tt > t ? 1u : 0u;
+        if (lead) {
+          if (tt == t_begin) trace_at(trace, 3);
           if (layout != kTwice) {   // one MMA per k-step (N = n_pad or 2 n_pad)
 #pragma unroll
             for (int kk = 0; kk < kTileK / 16; ++kk)
@@ -258,49 +238,38 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
             }
           }
           tc_commit(&ctl.empty[s]);
-          if (++s == S) {
-            s = 0;
-            ph ^= 1u;
-          }
         }
-        if (!ok) break;
-        tc_commit(&ctl.acc_full[buf]);
-        t = seg_end;
+        __syncwarp();
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      if (!ok) {  // tear-down: wait for every MMA already issued
-        tc_commit(&ctl.drain);
-        mbar_wait_drain(&ctl.drain, 0);
-      }
+      if (!ok) break;
+      if (lead) tc_commit(&ctl.acc_full[buf]);
+      __syncwarp();
+      t = seg_end;
+    }
+    if (!ok && lead) {  // tear-down: wait for every MMA already issued
+      tc_commit(&ctl.drain);
+      mbar_wait_drain(&ctl.drain, 0);
     }
   } else {
     // ------------------------------------------------ epilogue (warps 2-5)
     // a warp may only read TMEM lanes 32*(warp % 4) .. +31: that is its feature block
     const int ew = warp & 3;
     const int et = ew * 32 + lane;  // tile feature == TMEM lane
-    // cluster exchange: the first contributor of the row tile this range ends in
-    // expects its peers' partials (arrival count 1: this arrive; bytes may land first)
-    bool csk_reducer = false;
-    if (CSK && t_end > t_begin) {
-      const int rt_last = (t_end - 1) / KT;
-      const int cf = sk_cta_of(rt_last * KT, T, G), cl = sk_cta_of((rt_last + 1) * KT - 1, T, G);
-      csk_reducer = cf == c && cl > c && cf / a.csk == cl / a.csk;
-      if (csk_reducer && threadIdx.x == 64) {
-        mbar_arrive_expect_tx(&ctl.recv, static_cast<uint32_t>((cl - cf) * kTileM * 16 * 4));
-        ctl.recv_pending = 1;
-      }
-    }
     // the dry run overlaps the previous launch's tail; the real context follows
     // (ctx_early: the row plan is final before the wait, so the real context is
     // built there and the dry run uses it)
     if (a.ctx_early) {
       epi_prologue<EPI>(a, ectx, et);
-      if (a.warm) epilogue_warmup<EPI, CSK>(a, ectx, ctl.red, stage, rms, c, G, et, recv, csk_reducer);
+      if (a.warm) epilogue_warmup<EPI>(a, ectx, ctl.red, stage, rms, c, G, et);
     } else if (a.warm) {
       epi_ctx_dry(ectx, a.n_pad, et);
-      epilogue_warmup<EPI, CSK>(a, ectx, ctl.red, stage, rms, c, G, et, recv, csk_reducer);
+      epilogue_warmup<EPI>(a, ectx, ctl.red, stage, rms, c, G, et);
     }
     pdl_wait();
-    if constexpr (CSK) cluster_wait_acquire();
     if (threadIdx.x == 64) trace_at(trace, 13);
     if (a.rms) rms_prologue(a, rms, et);
     if (!a.ctx_early) epi_prologue<EPI>(a, ectx, et);
@@ -322,18 +291,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
       named_bar_sync(1, 128);
       if (!ok) break;
       tc_fence_after();
-      epilogue_segment<EPI, CSK>(a, ectx, layout, acols, tmem_base, buf, seg, c, G, rt, k0, k1, stage, rms,
-                       ctl.red, &ctl.reduce_flag, ctl.acc_empty, et, ew, lane, recv, &ctl.recv,
-                       abort_flag, threadIdx.x == 64 ? trace : nullptr);
+      epilogue_segment<EPI>(a, ectx, layout, acols, tmem_base, buf, seg, c, G, rt, k0, k1, stage, rms, ctl.red,
+                            &ctl.reduce_flag, ctl.acc_empty, et, ew, lane, threadIdx.x == 64 ? trace : nullptr);
       t = seg_end;
     }
   }
 
-  // a CTA that expects pushed partials leaves only after they landed (they do at
-  // once unless a peer stopped early; the wait is bounded)
-  if constexpr (CSK) {
-    if (threadIdx.x == 64 && ctl.recv_pending) mbar_wait_drain(&ctl.recv, 0);
-  }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -360,115 +323,39 @@ static int gemm_budget_bytes(int n_pad) {
   return n_pad <= 32 ? 200 * 1024 : 200 * 1024;
 }
 
-// Shared memory that receives the partials pushed by cluster peers: csk - 1
-// slots of one 128 x 16 fp32 accumulator each.
-static int csk_recv_bytes(int csk) { return csk > 1 ? (csk - 1) * kTileM * 16 * 4 + 16 : 0; }
-
-int gemm_pick_stages(int n_pad, int planes, int csk) {
+int gemm_pick_stages(int n_pad, int planes) {
   const int stage = kABytes + n_pad * 128 * planes;
   const int budget = gemm_budget_bytes(n_pad);
-  const int fixed = kTileM * kStagePitch * 4 + kMaxRows * 4 + static_cast<int>(sizeof(EpiCtx)) + 1024 +
-                    csk_recv_bytes(csk);
+  const int fixed = kTileM * kStagePitch * 4 + kMaxRows * 4 + static_cast<int>(sizeof(EpiCtx)) + 1024;
   int s = (budget - fixed) / stage;
   if (s > kMaxStages) s = kMaxStages;
   if (s < 2) s = 2;
   return s;
 }
 
-size_t gemm_smem_bytes(int n_pad, int stages, int planes, int csk) {
+size_t gemm_smem_bytes(int n_pad, int stages, int planes) {
   return static_cast<size_t>(stages) * (kABytes + n_pad * 128 * planes) + kTileM * kStagePitch * 4 +
-         kMaxRows * 4 + sizeof(EpiCtx) + 1024 + csk_recv_bytes(csk);
+         kMaxRows * 4 + sizeof(EpiCtx) + 1024;
 }
 
 cudaError_t gemm_set_max_smem() {
   // 227 KB per block minus the kernel's static shared memory
-  const void* fns[8] = {reinterpret_cast<const void*>(gemm_stream_kernel<EPI_F32, false>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_RESIDUAL, false>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_SWIGLU, false>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_QKV, false>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_F32, true>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_RESIDUAL, true>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_SWIGLU, true>),
-                        reinterpret_cast<const void*>(gemm_stream_kernel<EPI_QKV, true>)};
-  for (const void* f : fns) {
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-template <bool CSK>
-static const void* gemm_kernel_for(int epi) {
-  switch (epi) {
-    case EPI_F32: return reinterpret_cast<const void*>(gemm_stream_kernel<EPI_F32, CSK>);
-    case EPI_RESIDUAL: return reinterpret_cast<const void*>(gemm_stream_kernel<EPI_RESIDUAL, CSK>);
-    case EPI_SWIGLU: return reinterpret_cast<const void*>(gemm_stream_kernel<EPI_SWIGLU, CSK>);
-    case EPI_QKV: return reinterpret_cast<const void*>(gemm_stream_kernel<EPI_QKV, CSK>);
-    default: return nullptr;
-  }
-}
-
-int gemm_max_active_clusters(int epi, int csk, size_t smem) {
-  const void* fn = gemm_kernel_for<true>(epi);
-  if (fn == nullptr || csk < 2 || csk > 8) return 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(csk);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = csk;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
-  return n;
+  return cudaFuncSetAttribute(gemm_stream_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
 }
 
 cudaError_t launch_gemm(const GemmArgs& a, int grid, size_t smem, cudaStream_t s, bool pdl) {
+  if (a.epi != EPI_F32) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  int n_attr = 0;
-  if (pdl) {
-    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
-    ++n_attr;
-  }
-  if (a.csk > 1) {
-    if (a.csk > 8 || grid % a.csk != 0 || a.n_pad != 16) return cudaErrorInvalidValue;
-    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
-    attr[n_attr].val.clusterDim.x = a.csk;
-    attr[n_attr].val.clusterDim.y = 1;
-    attr[n_attr].val.clusterDim.z = 1;
-    ++n_attr;
-  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = n_attr;
-  if (a.csk > 1) {
-    switch (a.epi) {
-      case EPI_F32: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_F32, true>, a);
-      case EPI_RESIDUAL: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_RESIDUAL, true>, a);
-      case EPI_SWIGLU: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_SWIGLU, true>, a);
-      case EPI_QKV: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_QKV, true>, a);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (a.epi) {
-    case EPI_F32: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_F32, false>, a);
-    case EPI_RESIDUAL: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_RESIDUAL, false>, a);
-    case EPI_SWIGLU: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_SWIGLU, false>, a);
-    case EPI_QKV: return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_QKV, false>, a);
-    default: return cudaErrorInvalidValue;
-  }
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_F32>, a);
 }
 
 }  // namespace memspec

@@ -263,8 +263,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           mbar_wait_drain(ok ? &ctl.empty[q] : &ctl.full[q], (last_par >> q) & 1u);
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // ---------------------------------------------- CTA 0: MMAs
+      // The whole warp walks the tiles and one elected lane issues, so that descriptors
+      // and loop counters stay in uniform registers.
+      const bool lead = elect_one();
       const uint32_t idesc = make_idesc_bf16_f32(2 * kTileM, layout == kWide ? 2 * a.n_pad : a.n_pad);
       const uint64_t adesc0 = make_smem_desc_sw128(smem_addr(smem_a));
       const uint64_t bdesc0 = make_smem_desc_sw128(smem_addr(smem_b));
@@ -272,52 +275,52 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const uint32_t p_step = static_cast<uint32_t>(a.n_pad / 2 * 128) >> 4;   // kTwice: the lo plane
       int s = 0, seg = 0;
       uint32_t ph = 0;
-      bool ok = true, first = true;
+      bool ok = true;
       for (int t = t_begin; t < t_end && ok; ++seg) {
         const int seg_end = min(t_end, (t / KT + 1) * KT);
         const int buf = seg & 1;
-        if (seg >= 2 && !mbar_wait_cluster_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>((seg >> 1) - 1) & 1u,
-                                                   abort_flag, a.status)) {
-          ok = false;
-          break;
+        if (seg >= 2) {
+          ok = __all_sync(0xffffffffu,
+                          mbar_wait_cluster_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>((seg >> 1) - 1) & 1u,
+                                                    abort_flag, a.status));
+          if (!ok) break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * acols);
         for (int tt = t; tt < seg_end; ++tt) {
-          if (!mbar_wait_bounded(&ctl.full[s], ph, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          if (first) {
-            trace_at(trace, 3);
-            first = false;
-          }
+          ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.full[s], ph, abort_flag, a.status));
+          if (!ok) break;
           tc_fence_after();
           const uint64_t ad = adesc0 + static_cast<uint32_t>(s) * a_step;
           const uint64_t bd = bdesc0 + static_cast<uint32_t>(s) * b_step;
           const uint32_t acc0 = tt > t ? 1u : 0u;
-          if (layout != kTwice) {
+          if (lead) {
+            if (tt == t_begin) trace_at(trace, 3);
+            if (layout != kTwice) {
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk)
-              mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-          } else {
+              for (int kk = 0; kk < kTileK / 16; ++kk)
+                mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+            } else {
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk) {
-              mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-              mma_pair(d_tmem, ad + 2 * kk, bd + p_step + 2 * kk, idesc, 1u);
+              for (int kk = 0; kk < kTileK / 16; ++kk) {
+                mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+                mma_pair(d_tmem, ad + 2 * kk, bd + p_step + 2 * kk, idesc, 1u);
+              }
             }
+            commit_pair(&ctl.empty[s]);
           }
-          commit_pair(&ctl.empty[s]);
+          __syncwarp();
           if (++s == S) {
             s = 0;
             ph ^= 1u;
           }
         }
         if (!ok) break;
-        commit_pair(&ctl.acc_full[buf]);
+        if (lead) commit_pair(&ctl.acc_full[buf]);
+        __syncwarp();
         t = seg_end;
       }
-      if (!ok) {   // every MMA issued completes before the pair leaves
+      if (!ok && lead) {   // every MMA issued completes before the pair leaves
         commit_pair(&ctl.drain);
         mbar_wait_drain(&ctl.drain, 0);
       }

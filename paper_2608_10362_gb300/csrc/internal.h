@@ -15,6 +15,7 @@ typedef __nv_bfloat16 bf16;
 constexpr int kMaxGroups = 64;      // requests stepped together
 constexpr int kMaxRows = 256;       // rows of one forward pass (MMA N <= 256)
 constexpr int kPrefillChunk = 128;  // rows per prefill forward
+constexpr int kSmallRows = 8;       // rows (two planes) of a pass that runs gemm_small.cu
 constexpr int kMaxK = 15;           // largest draft length
 constexpr int kMaxDrafts = 16;
 constexpr int kStateInts = 4;       // per request: L, Lt, step, unused
@@ -142,9 +143,13 @@ struct GemmArgs {
   int split_epi;            // 1: contributors to a split row tile only store their partials;
                             // gemm_split_epi_kernel (the next launch) sums them and runs the
                             // epilogue, one CTA per (row tile, 16-row chunk)
+  int small;                // 1: gemm_small.cu's kernel (n_pad 16); x4d: 1: map_b, map_b2
+  int x4d;                  // are 4-D maps of the activations {64 columns, rows, planes, k tiles}
+                            // with boxes of one and of gemm_small_x_group k tiles; 0: 2-D maps
+                            // of the planes
   int pairs;                // > 0: gemm_pair.cu's kernel with this many CTA pairs (n_pad a
                             // = gemm_pair_pad, map_b boxes of gemm_pair_box_rows rows)
-  int csk;                  // > 1: launched in clusters of csk CTAs (n_pad == 16 only); a
+  int csk;                  // > 1: launched in clusters of csk CTAs (gemm_small.cu); a
                             // row tile whose contributors share a cluster is summed by
                             // its first contributor from partials the others push into
                             // its shared memory (no global partials, no counter)
@@ -338,13 +343,18 @@ cudaError_t launch_int4_pack(const uint8_t* qweight, const bf16* scales, const u
 // launchers (each returns the launch's cudaError_t)
 cudaError_t launch_embed(const EmbedArgs& a, int rows, cudaStream_t s, bool pdl);
 cudaError_t launch_gemm(const GemmArgs& a, int grid, size_t smem, cudaStream_t s, bool pdl);
-size_t gemm_smem_bytes(int n_pad, int stages, int planes = 1, int csk = 0);
-int gemm_pick_stages(int n_pad, int planes = 1, int csk = 0);
-// Thread-block clusters of `csk` CTAs of the GEMM kernel with epilogue `epi` and
-// `smem` bytes of dynamic shared memory that can be resident at once (0: none).
-int gemm_max_active_clusters(int epi, int csk, size_t smem);
+size_t gemm_smem_bytes(int n_pad, int stages, int planes = 1);
+int gemm_pick_stages(int n_pad, int planes = 1);
 cudaError_t gemm_set_max_smem();
 cudaError_t launch_gemm_split_epi(const GemmArgs& a, int gemm_grid, cudaStream_t s, bool pdl);
+// gemm_small.cu: ring stages, shared memory, thread-block clusters of csk CTAs that
+// can be resident at once (0: none), k tiles of a first-fill activation box
+int gemm_small_stages(int planes, int csk);
+size_t gemm_small_smem(int planes, int csk);
+int gemm_small_max_clusters(int epi, int planes, int csk);
+int gemm_small_x_group();
+cudaError_t gemm_small_set_max_smem();
+cudaError_t launch_gemm_small(const GemmArgs& a, int grid, cudaStream_t s, bool pdl);
 // gemm_pair.cu (stages, activation box rows and launch for n_pad rows in one plane
 // or, split, two)
 int gemm_pair_stages(int n_pad, int split, int epi);

@@ -22,6 +22,10 @@ def _bf16_pair(seed, rows, n_out, k):
 @pytest.mark.parametrize("rows,n_out,k", [
     (1, 256, 128), (5, 768, 256), (9, 688, 256), (16, 256, 688), (17, 2048, 2048),
     (6, 2560, 2048), (144, 1024, 4096), (128, 384, 352), (2, 640, 768), (256, 256, 256),
+    # up to 16 rows: one row tile, k of less than one, one and more than four k tiles, k not
+    # whole tiles, many row tiles per CTA, ranges that end inside a row tile
+    (16, 1, 8), (3, 128, 64), (9, 129, 328), (16, 300, 320), (1, 128, 4096), (7, 40000, 72), (8, 2560, 2048),
+    (13, 5000, 1000),
     # CTA pairs (from 161 rows): odd row tiles, one tile, ragged n and k, many tiles per pair
     (161, 129, 8), (161, 128, 64), (176, 300, 72), (193, 385, 4104), (255, 20001, 328), (256, 1, 1000),
 ])

@@ -155,11 +155,11 @@ def test_tiny_prompt_edge_cases(tiny):
         assert rep.band_flags == 0
 
 
-@pytest.mark.parametrize("B,K", [(2, 8), (3, 10), (8, 15), (9, 14), (10, 15), (16, 15)])
+@pytest.mark.parametrize("B,K", [(1, 1), (2, 3), (1, 8), (3, 3), (2, 8), (3, 10), (8, 15), (9, 14), (10, 15), (16, 15)])
 def test_verify_pass_row_counts(B, K):
-    """One verify pass at 18, 33, 128, 135, 160 and 256 rows (the CTA-pair GEMM's
-    operand layouts: two planes side by side up to 128 rows, one after the other
-    above), requests of different lengths: every request's logits and new K/V against
+    """One verify pass at 2, 8, 9, 12, 18, 33, 128, 135, 160 and 256 rows (up to 8: the
+    small GEMM; above: the CTA-pair GEMM's operand layouts, two planes side by side up
+    to 128 rows, one after the other above), requests of different lengths: every request's logits and new K/V against
     the oracle at the step tests' tolerance."""
     from oracle.llama import LlamaOracle
     from paper_2608_10362_gb300 import Engine, _lib
