@@ -43,7 +43,6 @@ __global__ void __launch_bounds__(kAttThreads, TQ ? 3 : 2) attn_kernel(const __g
     tma_prefetch_desc(&a.vmap);
   }
   __syncthreads();
-  pdl_launch_dependents();
   const int lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   unsigned long long* trace =
       (a.trace != nullptr && threadIdx.x == 0 && lin < a.trace_ctas) ? a.trace + lin * 16 : nullptr;
@@ -58,6 +57,7 @@ __global__ void __launch_bounds__(kAttThreads, TQ ? 3 : 2) attn_kernel(const __g
   if (a.tma && threadIdx.x == 0) fence_proxy_async_smem();
   auto wait = [&] {
     pdl_wait();
+    pdl_launch_dependents();
     trace_at(trace, 13);
   };
   const int kvh = blockIdx.y / a.row_blocks, rb = blockIdx.y - kvh * a.row_blocks;

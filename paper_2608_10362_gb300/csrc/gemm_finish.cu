@@ -81,7 +81,6 @@ gemm_split_epi_kernel(const __grid_constant__ GemmArgs a, int gemm_grid) {
   const int lin = blockIdx.y * gridDim.x + blockIdx.x;
   unsigned long long* ts = (a.trace != nullptr && et == 0 && lin < a.trace_ctas) ? a.trace + lin * 16 : nullptr;
   trace_at(ts, 0);
-  pdl_launch_dependents();
   // row tiles that a CTA owned whole were finished by it (gemm_pair.cu: with the
   // fp32-output epilogue only)
   if ((!a.pairs || EPI == EPI_F32) && c_first == c_last) return;
@@ -114,6 +113,7 @@ gemm_split_epi_kernel(const __grid_constant__ GemmArgs a, int gemm_grid) {
     }
   }
   if (a.ctx_early) pdl_wait();
+  pdl_launch_dependents();   // after the wait: see ptx.cuh
   trace_at(ts, 13);
   // ---- one round trip: sums of squares, residual rows, partials
   float ss = 0.f;

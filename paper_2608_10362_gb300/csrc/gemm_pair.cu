@@ -174,7 +174,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   // both CTAs' barriers and tensor memory exist before either touches the other's
   cluster_arrive_release();
   cluster_wait_acquire();
-  pdl_launch_dependents();
   const uint32_t tmem_base = ctl.tmem_base;
   unsigned long long* trace = a.trace != nullptr ? a.trace + blockIdx.x * 16 : nullptr;
   if (threadIdx.x == 64) trace_at(trace, 0);
@@ -229,6 +228,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         }
       }
       pdl_wait();
+      pdl_launch_dependents();   // after the wait: see ptx.cuh
       trace_at(trace, 2);
       for (int p = 0, k2 = kt_first; p < n_pre; ++p) {
         load_b(p, k2);

@@ -357,7 +357,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_small_kernel(const __grid_co
   // the barriers above are initialised before any peer pushes (every thread arrives
   // here; a thread waits before its first push)
   if constexpr (CSK) cluster_arrive_release();
-  pdl_launch_dependents();
   const uint32_t tmem_base = ctl.tmem_base;
   // optional trace (16 slots per CTA): 0 entry, 13 dependency released,
   // 2 activation loads issued, 3 first MMA, 4..12 epilogue, 1 exit
@@ -424,6 +423,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_small_kernel(const __grid_co
         next_tile();
       }
       pdl_wait();
+      pdl_launch_dependents();   // after the wait: see ptx.cuh
       trace_at(trace, 2);
       for (int p = 0, k2 = kt_first; p < n_pre;) {
         const int n = group_at(p, k2);
