@@ -947,7 +947,7 @@ def main():
     ap.add_argument("--launch-mode", default="per_op", choices=["per_op", "pass"],
                     help="one launch per op, or one persistent launch per pass")
     ap.add_argument("--draft-kernel", default="auto", choices=["auto", "per_op", "fused"],
-                    help="draft-step kernels (auto: the fused draft kernel when the draft fits it)")
+                    help="draft-step kernels (auto: the per-op kernels; fused: one launch per draft step)")
     ap.add_argument("--trace", default=None,
                     help="save per-op timestamps of the last traced pass (.npy); diagnostic, "
                          "not for the headline number")

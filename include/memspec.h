@@ -167,11 +167,11 @@ typedef struct memspec_init_params {
                                        1: verify passes, 2: draft steps, 3: prefill
                                        chunks (the last one); 0: off */
   int32_t draft_kernel;             /* draft step with launch_mode PER_OP:
-                                       MEMSPEC_DRAFT_KERNEL_AUTO (0): the fused draft
-                                       kernel when the draft and batch fit it (below),
-                                       else per-op kernels; PER_OP (1): always per-op
-                                       kernels; FUSED (2): the fused kernel, init or the
-                                       draft step fails with UNSUPPORTED if it cannot */
+                                       MEMSPEC_DRAFT_KERNEL_AUTO (0): the faster kernels,
+                                       which are the per-op ones for every draft and batch;
+                                       PER_OP (1): per-op kernels; FUSED (2): the whole step
+                                       as one launch, init or the draft step fails with
+                                       UNSUPPORTED if the draft or batch does not fit it */
 } memspec_init_params;
 
 enum { MEMSPEC_LAUNCH_PER_OP = 0, MEMSPEC_LAUNCH_PASS = 1 };

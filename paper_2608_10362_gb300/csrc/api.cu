@@ -641,8 +641,9 @@ memspec_status validate_params(const memspec_init_params* p, std::string* why) {
   return MEMSPEC_OK;
 }
 
-// Tensor map over a bf16 activation buffer [rows][cols] with box {64, n_pad}:
-// rows >= `rows` read as zero.  Cached per (buffer, rows, cols, n_pad).
+// Tensor map over a bf16 activation buffer or KV cache [rows][cols] with box {64,
+// n_pad}: rows >= `rows` read as zero.  Cached per (buffer, rows, cols, n_pad): a map
+// is a function of these alone.
 bool act_map(memspec_ctx* c, const void* ptr, int rows, int cols, int n_pad, CUtensorMap* out) {
   auto key = std::make_tuple(ptr, rows, cols, n_pad);
   auto it = c->bmaps.find(key);
@@ -663,8 +664,18 @@ bool pass_x(memspec_ctx* c, GemmArgs& a, bool pass, const bf16* hi, const bf16* 
     const long long apart = reinterpret_cast<const uint8_t*>(lo) - reinterpret_cast<const uint8_t*>(hi);
     if (rows <= kSmallRows && k % 64 == 0 && apart > 0) {
       a.x4d = 1;
-      return encode_x4(&a.map_b, hi, rows, k, 2, apart, 8, 1) &&
-             encode_x4(&a.map_b2, hi, rows, k, 2, apart, 8, gemm_small_x_group());
+      auto map = [&](int box_kt, CUtensorMap* out) {   // the planes of a buffer have one distance
+        const auto key = std::make_tuple(static_cast<const void*>(hi), rows, k, -box_kt);
+        auto it = c->bmaps.find(key);
+        if (it == c->bmaps.end()) {
+          CUtensorMap m;
+          if (!encode_x4(&m, hi, rows, k, 2, apart, 8, box_kt)) return false;
+          it = c->bmaps.emplace(key, m).first;
+        }
+        *out = it->second;
+        return true;
+      };
+      return map(1, &a.map_b) && map(gemm_small_x_group(), &a.map_b2);
     }
     box = rows <= kSmallRows ? 8 : gemm_pair_box_rows(n_pad, 1);
   }
@@ -949,8 +960,8 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       // per-op launches stream K/V tiles by TMA (the persistent pass kernel keeps cp.async)
       if (!pass) {
         const int kv_rows = c->p.max_batch * cf.n_kv_heads * c->p.max_seq;
-        if (!encode_map(&at.kmap, kl, kv_rows, cf.head_dim, 64) ||
-            !encode_map(&at.vmap, vl, kv_rows, cf.head_dim, 64))
+        if (!act_map(c, kl, kv_rows, cf.head_dim, 64, &at.kmap) ||
+            !act_map(c, vl, kv_rows, cf.head_dim, 64, &at.vmap))
           return fail(c, MEMSPEC_ERR_CUDA, "KV tensor map");
         at.tma = 1;
       }
@@ -1218,6 +1229,13 @@ memspec_status run_pass(memspec_ctx* c, const GraphKey& key, bool use_pass, Emit
     if (s != MEMSPEC_OK) return s;
   }
   if (!c->p.use_graphs) return pass ? launch_table(c, t) : run_ops_separately(c, ops);
+  // The first use runs as plain launches and is captured for the next ones while the
+  // GPU is at work: capturing 250 launches before the first of them runs would hold a
+  // request's first step for a millisecond.
+  if (!pass) {
+    s = run_ops_separately(c, ops);
+    if (s != MEMSPEC_OK) return s;
+  }
   cudaError_t e = cudaStreamBeginCapture(c->main, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(c, e, "begin capture");
   s = pass ? launch_table(c, t) : run_ops_separately(c, ops);
@@ -1234,6 +1252,7 @@ memspec_status run_pass(memspec_ctx* c, const GraphKey& key, bool use_pass, Emit
   if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
   c->graphs.emplace(key, ex);
   c->graph_launches[key] = n_launch;
+  if (!pass) return MEMSPEC_OK;
   e = cudaGraphLaunch(ex, c->main);
   if (e != cudaSuccess) return cuda_fail(c, e, "graph launch");
   return MEMSPEC_OK;
@@ -1844,16 +1863,17 @@ memspec_status memspec_draft_step(memspec_ctx* c, int32_t K, float T) {
   if (s != MEMSPEC_OK) return s;
   const int B = c->batch;
   const int id = c->active;
-  if (!c->pass_kernel && c->p.draft_kernel != MEMSPEC_DRAFT_KERNEL_PER_OP) {
+  // The fused kernel runs on request only: one launch of grid-wide phases took less
+  // time than per-op launches while those were 8 to 10 us each, but not since
+  // gemm_small.cu (160M draft, K = 4, context 2048: 1.52 ms against 1.32; four requests
+  // 2.98 / 1.47; 68M, K = 5, context 512: 0.425 / 0.317).
+  if (!c->pass_kernel && c->p.draft_kernel == MEMSPEC_DRAFT_KERNEL_FUSED) {
     DraftFusedArgs fa{};
     std::string why;
-    const bool fits = fused_draft_plan(c, d, K, T, &fa, &why);
-    if (fits) {
-      c->last_draft_fused = true;
-      return run_fused_draft(c, GraphKey{3, id, K, fbits(T), B}, fa);
-    }
-    if (c->p.draft_kernel == MEMSPEC_DRAFT_KERNEL_FUSED)
+    if (!fused_draft_plan(c, d, K, T, &fa, &why))
       return fail(c, MEMSPEC_ERR_UNSUPPORTED, "fused draft kernel: " + why);
+    c->last_draft_fused = true;
+    return run_fused_draft(c, GraphKey{3, id, K, fbits(T), B}, fa);
   }
   c->last_draft_fused = false;
   GraphKey key{0, id, K, fbits(T), B};

@@ -1,4 +1,5 @@
-// draft_fused.cu - the draft step of a small draft model as ONE launch.
+// draft_fused.cu - the draft step of a small draft model as ONE launch (init param
+// draft_kernel = FUSED; the per-op kernels are faster, see memspec_draft_step).
 //
 // The draft step is K autoregressive forward passes of one position each (two
 // for the first pass after a fully accepted step) plus a categorical sample per

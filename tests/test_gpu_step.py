@@ -62,6 +62,30 @@ def test_tiny_pair_lockstep(tiny, T, mode):
     assert list(eng.committed_tokens(0)) == sd.tokens
 
 
+@pytest.mark.parametrize("B", [1, 4])
+@pytest.mark.parametrize("T", [0.0, 1.0])
+def test_tiny_pair_lockstep_fused_draft_kernel(tiny, T, B):
+    """The draft step as one launch (draft_kernel "fused"), one and four requests."""
+    from paper_2608_10362_gb300 import _lib
+    _, to, do, (t, wt, d, wd) = tiny
+    eng = _engine(t, wt, d, wd, True, "per_op", max_batch=B, draft_kernel="fused")
+    prompts = [gen_prompt(27 + b, 100 + 9 * b, 2048) for b in range(B)]
+    sds = []
+    for b, p in enumerate(prompts):
+        eng.prefill(b, p, seed=5 + b)
+        sds.append(SpecDecoder(to, do, p, 256))
+    eng.set_batch(B)
+    rep = LockstepReport()
+    for step in range(6):
+        eng.step(4, T, eng.results_host)
+        for b in range(B):
+            check_step(eng, sds[b], 4, T, 5 + b, step, rep, req=b, batch=B)
+    assert eng.info(_lib.INFO_DRAFT_FUSED) == 1
+    line = rep.record(f"tiny fused draft kernel T={T} B={B}")
+    eng.close()
+    assert rep.band_flags == 0, line
+
+
 def test_tiny_pair_lockstep_per_op_draft_path(tiny):
     """The draft step through the per-op kernels (the path larger drafts take),
     T = 1."""
