@@ -835,15 +835,12 @@ memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, bool pass, std::vector<Pas
   return MEMSPEC_OK;
 }
 
-// Launches as separate kernels: the op after the embedding kernel (which writes
-// the row plan) waits for every earlier kernel (no programmatic dependent
-// launch), so every later op starts after the plan - and the KV cache of earlier
-// positions - is final and may read them before griddepcontrol.wait (ctx_early).
-// MEMSPEC_CTX_EARLY=0 turns this off (measurement).
+// Launches as separate kernels: a kernel of a pass lets the next one start only after
+// its own griddepcontrol.wait, so when the op two after the embedding kernel (which
+// writes the row plan) starts, the embedding kernel has completed: the plan - and the
+// KV cache of earlier positions - is final for it and every later op, which may read
+// them before their wait (ctx_early).
 void mark_ctx_early(std::vector<PassOp>& ops, size_t first) {
-  static const int enabled = env_int("MEMSPEC_CTX_EARLY", 1);
-  if (!enabled || ops.size() < first + 2 || ops[first].type != OP_EMBED) return;
-  ops[first + 1].full_dep = 1;
   for (size_t i = first + 2; i < ops.size(); ++i) {
     if (ops[i].type == OP_GEMM || ops[i].type == OP_GEMM_EPI) ops[i].u.g.ctx_early = 1;
     if (ops[i].type == OP_ATTN) ops[i].u.at.ctx_early = 1;
@@ -1090,11 +1087,11 @@ memspec_status run_ops_separately(memspec_ctx* c, const std::vector<PassOp>& ops
     switch (op.type) {
       case OP_EMBED: e = launch_embed(op.u.e, op.n_units, c->main, c->pdl); break;
       case OP_GEMM:
-        e = op.u.g.pairs ? launch_gemm_pair(op.u.g, c->main, c->pdl && !op.full_dep)
-                         : launch_gemm_small(op.u.g, op.grid, c->main, c->pdl && !op.full_dep);
+        e = op.u.g.pairs ? launch_gemm_pair(op.u.g, c->main, c->pdl)
+                         : launch_gemm_small(op.u.g, op.grid, c->main, c->pdl);
         break;
       case OP_GEMM_EPI: e = launch_gemm_split_epi(op.u.g, op.grid, c->main, c->pdl); break;
-      case OP_ATTN: e = launch_attention(op.u.at, op.grid, c->main, c->pdl && !op.full_dep); break;
+      case OP_ATTN: e = launch_attention(op.u.at, op.grid, c->main, c->pdl); break;
       case OP_SAMPLE: e = launch_sample(op.u.s, c->main, c->pdl); break;
       case OP_ACCEPT: e = launch_accept(op.u.acc, c->main, false); break;
       case OP_TREE_WALK: e = launch_tree_walk(op.u.tw, c->main); break;

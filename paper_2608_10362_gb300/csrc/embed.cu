@@ -20,8 +20,8 @@ namespace {
 // one CTA per row
 __global__ void __launch_bounds__(256) embed_kernel(const __grid_constant__ EmbedArgs a) {
   __shared__ float red[8];
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   emb::embed_row<256>(a, blockIdx.x, red, threadIdx.x, [] { __syncthreads(); });
 }
 

@@ -180,9 +180,8 @@ struct GemmArgs {
   int trace_ctas;           // split epilogue kernel: CTAs (linear index) that record
   int warm;                 // 1: dry run of the tail before griddepcontrol.wait
   int ctx_early;            // 1: every kernel before the previous one has completed when
-                            // this one starts (an earlier launch of the pass had a full
-                            // dependency after the row-plan writer), so the row plan
-                            // may be read before griddepcontrol.wait
+                            // this one starts and the row-plan writer is among them, so
+                            // the row plan may be read before griddepcontrol.wait
 };
 
 struct AttnArgs {

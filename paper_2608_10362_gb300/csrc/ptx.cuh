@@ -148,7 +148,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // CTAs were handed out while an earlier kernel still held part of the chip, and some
 // of them started 6 us late although SMs were free by then (verify pass of the 1.1B
 // target 0.866 -> 0.821 ms, 7B 2.755 -> 2.715, batched 8B 7.25 -> 7.12).  One launch's
-// time is still enough for the next one's set-up and first copies.
+// time is still enough for the next one's set-up and first copies.  It also means that
+// when a kernel starts, the one before its predecessor has completed.
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
     }
     cluster_arrive_release();   // waited for before the first push
   }
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   const Slice s = slice_of(a, g, rank, C);
   const int off0 = s.base + w * kTileIds + lane * 4;
   float best = -INFINITY;
