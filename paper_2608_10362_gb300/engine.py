@@ -8,6 +8,7 @@ the library reports (memspec_weights_offset), and forwards calls.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 from typing import Iterable, Mapping
 
 import numpy as np
@@ -344,21 +345,42 @@ def _as_triples(weights):
 
 
 # ------------------------------------------------------------------ op-level calls
+# These wrap one or two kernel launches of a few microseconds, so the wrapper's own
+# time counts: the stream is read as a raw handle, and what is a function of sizes
+# alone is remembered by size.
+def _raw_stream(x: torch.Tensor, stream) -> int:
+    """cudaStream_t of `stream`, else of the current stream of x's device."""
+    if stream is not None:
+        return stream.cuda_stream
+    dev = x.get_device()
+    if dev < 0:
+        return torch.cuda.current_stream(x.device).cuda_stream   # not a CUDA tensor: raises
+    return torch._C._cuda_getCurrentRawStream(dev)
+
+
+@functools.lru_cache(maxsize=512)
+def _linear_scratch_bytes(rows: int, n_out: int, k: int) -> int:
+    lib = _lib.load()
+    nb = C.c_size_t()
+    _check(lib, lib.memspec_op_linear_scratch_bytes(rows, n_out, k, C.byref(nb)))
+    return nb.value
+
+
 def op_linear(x: torch.Tensor, w: torch.Tensor, scratch: torch.Tensor | None = None,
               stream: torch.cuda.Stream | None = None) -> torch.Tensor:
-    """y = x . w^T on the weight-streaming GEMM kernel (x, w bf16 on cuda)."""
+    """y = x . w^T on the weight-streaming GEMM kernels (x, w bf16 on cuda)."""
     lib = _lib.load()
     rows, k = x.shape
     n_out = w.shape[0]
-    nb = C.c_size_t()
-    _check(lib, lib.memspec_op_linear_scratch_bytes(rows, n_out, k, C.byref(nb)))
+    nb = _linear_scratch_bytes(rows, n_out, k)
     if scratch is None:
-        scratch = torch.zeros(nb.value + 256, dtype=torch.uint8, device=x.device)
-    base = (scratch.data_ptr() + 255) // 256 * 256
-    y = torch.empty(rows, n_out, dtype=torch.float32, device=x.device)
-    s = stream or torch.cuda.current_stream(x.device)
-    _check(lib, lib.memspec_op_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, n_out, k,
-                                      base, nb.value, None, s.cuda_stream))
+        scratch = torch.zeros(nb + 256, dtype=torch.uint8, device=x.device)
+    base = (scratch.data_ptr() + 255) & ~255
+    y = torch.empty((rows, n_out), dtype=torch.float32, device=x.device)
+    st = lib.memspec_op_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, n_out, k, base, nb, None,
+                               _raw_stream(x, stream))
+    if st:
+        _check(lib, st)
     return y
 
 
@@ -373,12 +395,11 @@ def op_linear_noalloc(x: torch.Tensor, w: torch.Tensor, y: torch.Tensor | None =
     rows, k = x.shape
     n_out = w.shape[0]
     if y is None:
-        y = torch.empty(rows, n_out, dtype=torch.float32, device=x.device)
-    s = stream or torch.cuda.current_stream(x.device)
-    _check(lib, lib.memspec_op_linear_noalloc(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows,
-                                              n_out, k,
-                                              None if status is None else status.data_ptr(),
-                                              s.cuda_stream))
+        y = torch.empty((rows, n_out), dtype=torch.float32, device=x.device)
+    st = lib.memspec_op_linear_noalloc(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, n_out, k,
+                                       None if status is None else status.data_ptr(), _raw_stream(x, stream))
+    if st:
+        _check(lib, st)
     return y
 
 
@@ -394,9 +415,8 @@ def int4_pack(qweight: torch.Tensor, scales: torch.Tensor, zeros: torch.Tensor,
     if nbytes < 0:
         raise MemSpecError(_lib.ERR_INVALID_ARG, f"bad INT4 shape n={n_out} k={k}")
     packed = torch.empty(nbytes, dtype=torch.uint8, device=qweight.device)
-    s = stream or torch.cuda.current_stream(qweight.device)
     _check(lib, lib.memspec_int4_pack(qweight.data_ptr(), scales.data_ptr(), zeros.data_ptr(), n_out, k,
-                                      packed.data_ptr(), s.cuda_stream))
+                                      packed.data_ptr(), _raw_stream(qweight, stream)))
     return packed
 
 
@@ -409,19 +429,20 @@ def op_linear_int4(x: torch.Tensor, packed: torch.Tensor, n_out: int, y: torch.T
     lib = _lib.load()
     rows, k = x.shape
     if y is None:
-        y = torch.empty(rows, n_out, dtype=torch.float32, device=x.device)
-    s = stream or torch.cuda.current_stream(x.device)
-    _check(lib, lib.memspec_op_linear_int4(x.data_ptr(), packed.data_ptr(), y.data_ptr(), rows, n_out, k,
-                                           None if status is None else status.data_ptr(), s.cuda_stream))
+        y = torch.empty((rows, n_out), dtype=torch.float32, device=x.device)
+    st = lib.memspec_op_linear_int4(x.data_ptr(), packed.data_ptr(), y.data_ptr(), rows, n_out, k,
+                                    None if status is None else status.data_ptr(), _raw_stream(x, stream))
+    if st:
+        _check(lib, st)
     return y
 
 
 def op_sample(logits: torch.Tensor, temperature: float, u: torch.Tensor | None = None):
     lib = _lib.load()
     rows, vocab = logits.shape
-    out = torch.empty(rows, dtype=torch.int32, device=logits.device)
-    s = torch.cuda.current_stream(logits.device)
-    _check(lib, lib.memspec_op_sample(logits.data_ptr(), rows, vocab, C.c_float(temperature),
-                                      None if u is None else u.data_ptr(), out.data_ptr(),
-                                      s.cuda_stream))
+    out = torch.empty((rows,), dtype=torch.int32, device=logits.device)
+    st = lib.memspec_op_sample(logits.data_ptr(), rows, vocab, temperature,
+                               None if u is None else u.data_ptr(), out.data_ptr(), _raw_stream(logits, None))
+    if st:
+        _check(lib, st)
     return out
