@@ -2289,7 +2289,8 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
     maps = a.x4d ? encode_x4(&a.map_b, x, rows, k, 1, static_cast<long long>(k) * 2, 16, 1) &&
                        encode_x4(&a.map_b2, x, rows, k, 1, static_cast<long long>(k) * 2, 16, gemm_small_x_group())
                  : encode_map(&a.map_b, x, rows, k, 16);
-    if (maps) e = launch_gemm_small(a, grid, st, false);
+    a.w_after_wait = 1;
+    if (maps) e = launch_gemm_small(a, grid, st, true);   // set-up overlaps the previous kernel's end
   } else {
     a.pairs = gemm_pairs(rows, 0, a.row_tiles, a.k_tiles);
     a.n_pad = a.pairs ? gemm_pair_pad(rows, 0) : n_pad;
@@ -2405,7 +2406,7 @@ memspec_status memspec_op_sample(const float* logits, int32_t rows, int32_t voca
   sa.u_explicit = u;
   sa.out_tok = out;
   sa.out_stride = 1;
-  cudaError_t e = launch_sample(sa, static_cast<cudaStream_t>(stream), false);
+  cudaError_t e = launch_sample(sa, static_cast<cudaStream_t>(stream), true);
   if (e != cudaSuccess) {
     g_op_error = std::string("sample launch: ") + cudaGetErrorString(e);
     return MEMSPEC_ERR_CUDA;

@@ -23,8 +23,10 @@
 //   7B target, 5 rows    QKV 21.8 / 16.4 (6.1 TB/s), O 14.5 / 7.7, gate/up 31.0 / 28.2
 //                        (6.4 TB/s), down 20.0 / 15.4; verify pass 3.28 / 2.73 ms
 //   1.1B target, 6 rows  QKV 10.5 / 4.6, O 10.5 / 5.2, down 14.3 / 7.9; 1.31 / 0.90 ms
-//   alone, 5 rows        2304 x 768 8.5 / 5.6, 4096 x 4096 13.9 / 10.1, 28672 x 4096 44.5 /
-//                        39.3 (6.0 TB/s)
+//   alone, 5 rows        2304 x 768 8.5 / 4.2, 4096 x 4096 13.9 / 8.6, 28672 x 4096 44.5 /
+//                        38.2 (6.2 TB/s); without the launch overlapping the previous one's
+//                        end (set-up, dry run; every read stays behind the wait) 5.6, 10.1,
+//                        39.3
 // Tried instead: the features of a launch dealt to CTAs in any number over all of k,
 // without split-K (mma.sync from registers or from row runs of the packed tiles): 2 to 3
 // TB/s, a run of 27 rows is 3.4 KB a k tile.
@@ -410,6 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_small_kernel(const __grid_co
       // before the wait (a group's activations complete on its first stage's barrier:
       // stages are read in order)
       const int kt_first = kt;
+      if (a.w_after_wait) pdl_wait();
       for (int p = 0, left = 0; p < n_pre; ++p) {
         uint32_t bytes = kABytes;
         if (left == 0) {

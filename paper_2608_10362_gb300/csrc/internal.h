@@ -147,6 +147,9 @@ struct GemmArgs {
   int x4d;                  // are 4-D maps of the activations {64 columns, rows, planes, k tiles}
                             // with boxes of one and of gemm_small_x_group k tiles; 0: 2-D maps
                             // of the planes
+  int w_after_wait;         // gemm_small.cu, 1: the weights too are read only after
+                            // griddepcontrol.wait (an op-level call's weights may be anything
+                            // that earlier work on the stream writes)
   int pairs;                // > 0: gemm_pair.cu's kernel with this many CTA pairs (n_pad a
                             // = gemm_pair_pad, map_b boxes of gemm_pair_box_rows rows)
   int csk;                  // > 1: launched in clusters of csk CTAs (gemm_small.cu); a

@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(kSThreads) accept_kernel(const __grid_constant
 // CTAs per row and float4 per thread and round (2 or 8).  A row is cut in two while
 // the launch's CTAs still fit the chip at two per SM and a CTA keeps 2048 ids.
 // Measured (GB300, kernel alone, T = 1; before: one CTA per row, which read its row
-// twice): 1 x 32000 18.5 -> 3.8 us, 1 x 128256 57.5 -> 5.5, 32 x 128256 75.8 -> 8.9,
-// 144 x 128256 77.3 -> 21.8 (3.4 TB/s), 256 x 128256 101 -> 37.5.  Clusters of eight
+// twice): 1 x 32000 18.5 -> 3.3 us, 1 x 128256 57.5 -> 5.0, 32 x 128256 75.8 -> 8.3,
+// 144 x 128256 77.3 -> 20.9 (3.5 TB/s), 256 x 128256 101 -> 37.  Clusters of eight
 // whatever the row count: 144 x 128256 36 us (four waves of short CTAs); a
 // persistent grid that copies its next row while it reduces one: 35 us.
 struct SampleShape {
