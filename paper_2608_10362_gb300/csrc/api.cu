@@ -82,6 +82,20 @@ bool encode_x4(CUtensorMap* map, const void* base, int rows, int k, int planes, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// K or V cache of a layer, [rows][hd] bf16, in boxes of 128 rows by all of hd: two 64
+// column halves one after the other, each with the 128-byte swizzle.
+bool encode_kv(CUtensorMap* map, const void* base, long long rows, int hd) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (fn == nullptr || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
+  cuuint64_t dims[3] = {64, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(hd / 64)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(hd) * 2, 128};
+  cuuint32_t box[3] = {64, 128, static_cast<cuuint32_t>(hd / 64)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Packed tiles (16 KB each, contiguous) as rows of 256 bf16, box {256, 32}: one tile
 // per box, copied as stored.
 bool encode_packed(CUtensorMap* map, const void* base, long long tiles) {
@@ -148,6 +162,7 @@ bool ensure_func_attrs() {
     return false;
   }
   e = attention_set_max_smem();
+  if (e == cudaSuccess) e = attn_tc_set_max_smem();
   if (e != cudaSuccess) {
     g_attr_error = std::string("attention smem attribute: ") + cudaGetErrorString(e);
     return false;
@@ -261,11 +276,10 @@ struct AttnGeo {
 AttnGeo attn_geometry(const memspec_model_cfg& c, int groups, int R, int max_seq) {
   AttnGeo g;
   const int gs = c.n_heads / c.n_kv_heads;
-  // query vectors per CTA: at most 64 (4 m-tiles of 16); decode-sized GQA passes
-  // (2..8 query heads per KV head, at most 64 vectors in all) take row blocks of
-  // at most 8 vectors for the transposed form - every warp busy, three CTAs per
-  // SM; the blocks of a head re-read its keys, mostly from L2 (batched 8B verify,
-  // 36 vectors per head: 11.0 -> 9.8 ms)
+  // query vectors per CTA: at most 64 (4 m-tiles of 16; the persistent pass kernel);
+  // decode-sized GQA passes (2..8 query heads per KV head, at most 64 vectors in all)
+  // take row blocks of at most 8 vectors; the blocks of a head re-read its keys, mostly
+  // from L2
   const int qlimit = (gs >= 2 && gs <= 8 && gs * R <= 64) ? 8 : 64;
   int rpb = std::max(1, qlimit / gs);
   rpb = std::min(rpb, R);
@@ -274,10 +288,10 @@ AttnGeo attn_geometry(const memspec_model_cfg& c, int groups, int R, int max_seq
   g.qmax = gs * rpb;
   const int units = groups * c.n_kv_heads * g.row_blocks;
   const int max_splits = ceil_div(max_seq, 64);
-  // one wave of CTAs: the transposed form (at most 8 query vectors per CTA, 2
-  // stages) fits three per SM, the 16-row form (3 stages) two (an extra partial
-  // wave would double the time); at most 16 splits (the combine fetches 16
-  // splits' outputs per round trip)
+  // one wave of CTAs (an extra partial wave would double the time): the transposed
+  // form (attention.cu: at most 8 query vectors per CTA, 2 stages) fits three per SM,
+  // the 16-row form (the pass kernel) was sized for two; at most 16 splits (the combine
+  // fetches 16 splits' outputs per round trip)
   const bool tq = g.qmax <= 8;
   const int per_sm = tq ? 3 : 2;
   int want = std::max(1, std::min(16, (per_sm * sm_count()) / units));
@@ -291,6 +305,43 @@ AttnGeo attn_geometry(const memspec_model_cfg& c, int groups, int R, int max_seq
     g.chunk *= 2;
     g.n_splits = ceil_div(max_seq, g.chunk);
   }
+  return g;
+}
+
+// attn_tc.cu's launch for a pass, cluster 0: attention.cu's kernel.
+struct AttnTcGeo {
+  int rows_per_block, row_blocks, qmax, cluster;
+};
+// The cluster that shares a unit's keys is the largest whose launch is resident at once
+// and has a tile of keys per CTA (4 draft rows at 3000 keys, 12 units, 8 layers: 8 CTAs
+// 0.215 ms, 4 0.235, 2 0.279; 16 units of the 1.1B at 3000 keys: 4 CTAs 0.330, 8, in
+// two waves, 0.379).  attention.cu's kernel keeps passes of at most 8 query vectors per
+// KV head in units too many for clusters of four, where its three small CTAs per SM read
+// faster than one (8 layers, ms, this kernel / that): 7B, 4 requests x 5 rows, 3000 keys
+// 1.043 / 1.018; 160M, 16 x 5 rows, 3000 keys 0.732 / 0.596; 8B, 16 x 2 rows, 3000 keys
+// 1.192 / 1.162 - but 7B, 1 x 5 rows, 700 keys 0.667 / 0.692; 8B, 4 x 2 rows, 700 keys
+// 0.827 / 0.854; 7B, 4 x 9 rows, 700 keys 0.856 / 0.905.
+AttnTcGeo attn_tc_geometry(const memspec_model_cfg& c, int groups, int R, int max_keys) {
+  AttnTcGeo g{};
+  const int gs = c.n_heads / c.n_kv_heads;
+  g.rows_per_block = std::max(1, std::min(R, 128 / gs));
+  g.row_blocks = ceil_div(R, g.rows_per_block);
+  g.qmax = std::min(128, gs * g.rows_per_block);
+  const int units = groups * c.n_kv_heads * g.row_blocks;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  static std::map<std::tuple<int, int, int, int>, int> fit;   // (device, hd, qmax, C) -> clusters
+  static std::mutex fit_mu;
+  std::lock_guard<std::mutex> lock(fit_mu);
+  g.cluster = 1;
+  for (int C = 2; C <= 8 && (C / 2) * 128 < max_keys; C *= 2) {
+    const auto key = std::make_tuple(dev, c.head_dim, g.qmax, C);
+    auto it = fit.find(key);
+    if (it == fit.end()) it = fit.emplace(key, attn_tc_max_clusters(c.head_dim, g.qmax, C)).first;
+    if (units > it->second) break;
+    g.cluster = C;
+  }
+  if (gs * R <= 8 && g.cluster < 4) g.cluster = 0;
   return g;
 }
 
@@ -895,6 +946,9 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
   if (attn_part_floats(cf, geo, f.n_groups) > c->att_po_cap ||
       attn_units(cf, geo, f.n_groups) > c->att_cnt_cap)
     return fail(c, MEMSPEC_ERR_UNSUPPORTED, "attention partial buffer too small for this pass");
+  const AttnTcGeo tc =
+      pass ? AttnTcGeo{}
+           : attn_tc_geometry(cf, f.n_groups, f.R, f.mode == PLAN_PREFILL ? f.pre_start + f.pre_count : c->p.max_seq);
   int ss_count = 1;
   for (int l = 0; l < cf.n_layers; ++l) {
     bf16* kl = m.kv + static_cast<size_t>(l) * 2 * layer_kv;
@@ -957,7 +1011,15 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       // per-op launches stream K/V tiles by TMA (the persistent pass kernel keeps cp.async)
       if (!pass) {
         const int kv_rows = c->p.max_batch * cf.n_kv_heads * c->p.max_seq;
-        if (!act_map(c, kl, kv_rows, cf.head_dim, 64, &at.kmap) ||
+        if (tc.cluster > 0) {
+          at.tc = 1;
+          at.rows_per_block = tc.rows_per_block;
+          at.row_blocks = tc.row_blocks;
+          at.n_splits = tc.cluster;
+          at.qmax = tc.qmax;
+          if (!encode_kv(&at.kmap, kl, kv_rows, cf.head_dim) || !encode_kv(&at.vmap, vl, kv_rows, cf.head_dim))
+            return fail(c, MEMSPEC_ERR_CUDA, "KV tensor map");
+        } else if (!act_map(c, kl, kv_rows, cf.head_dim, 64, &at.kmap) ||
             !act_map(c, vl, kv_rows, cf.head_dim, 64, &at.vmap))
           return fail(c, MEMSPEC_ERR_CUDA, "KV tensor map");
         at.tma = 1;
@@ -1091,7 +1153,10 @@ memspec_status run_ops_separately(memspec_ctx* c, const std::vector<PassOp>& ops
                          : launch_gemm_small(op.u.g, op.grid, c->main, c->pdl);
         break;
       case OP_GEMM_EPI: e = launch_gemm_split_epi(op.u.g, op.grid, c->main, c->pdl); break;
-      case OP_ATTN: e = launch_attention(op.u.at, op.grid, c->main, c->pdl); break;
+      case OP_ATTN:
+      e = op.u.at.tc ? launch_attn_tc(op.u.at, op.grid, c->main, c->pdl)
+                     : launch_attention(op.u.at, op.grid, c->main, c->pdl);
+      break;
       case OP_SAMPLE: e = launch_sample(op.u.s, c->main, c->pdl); break;
       case OP_ACCEPT: e = launch_accept(op.u.acc, c->main, false); break;
       case OP_TREE_WALK: e = launch_tree_walk(op.u.tw, c->main); break;

@@ -90,7 +90,7 @@ __host__ __device__ constexpr size_t attention_smem_bytes_hd() {
 
 // One CTA of split-KV attention for unit (g, kvh, rb, split), run by 128 threads
 // (tid 0..127); `sync` is a barrier over exactly those threads; smem_raw is the
-// CTA's attention shared memory (attention_smem_bytes).  Returns early, all
+// CTA's attention shared memory (attention_smem_bytes_hd).  Returns early, all
 // threads together, when the unit has no work.
 // dry: a run of the same code on one synthetic tile that reads only scratch and
 // writes no global memory (no output, no partials, no counters): launched

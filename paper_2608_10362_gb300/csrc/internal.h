@@ -190,6 +190,8 @@ struct GemmArgs {
 struct AttnArgs {
   CUtensorMap kmap;         // tma: this layer's K cache as [max_batch * Hkv * max_seq][hd] bf16,
   CUtensorMap vmap;         //   box {64, 64}, 128-byte swizzle; V likewise
+  int tc;                   // 1: attn_tc.cu's kernel: the maps' boxes are {64, 128, hd / 64},
+                            //   n_splits is the cluster's size; partials and counters unused
   int tma;                  // 1: K/V tiles by cp.async.bulk.tensor into mbarrier stages
   const float* q;           // [rows][H][hd] fp32, rotated
   const bf16* kcache;       // [req][Hkv][max_seq][hd]
@@ -365,8 +367,11 @@ int gemm_pair_box_rows(int n_pad, int split);
 cudaError_t gemm_pair_set_max_smem();
 cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_attention(const AttnArgs& a, int n_groups, cudaStream_t s, bool pdl);
-size_t attention_smem_bytes(const AttnArgs& a);
 cudaError_t attention_set_max_smem();
+cudaError_t attn_tc_set_max_smem();
+// Clusters of C CTAs of the kernel for at most qmax vectors that fit the device at once.
+int attn_tc_max_clusters(int hd, int qmax, int C);
+cudaError_t launch_attn_tc(const AttnArgs& a, int n_groups, cudaStream_t s, bool pdl);
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_rope_table(float* cos_t, float* sin_t, int max_seq, int half, float base,

@@ -215,3 +215,36 @@ def test_verify_pass_row_counts(B, K):
             assert np.abs(got - k_ref).max() <= 2.0 ** -7 * np.abs(k_ref).max()
     finally:
         eng.close()
+
+
+@pytest.mark.parametrize("H,Hkv,hd,K", [(2, 2, 64, 1), (16, 2, 64, 3), (16, 2, 64, 4), (16, 2, 64, 7), (16, 2, 64, 8),
+                                        (16, 2, 64, 15), (1, 1, 128, 8), (4, 1, 128, 8), (12, 1, 128, 10)])
+@pytest.mark.parametrize("lens", [(3,), (120, 128, 129), (1100, 30)])
+def test_attention_of_many_vectors(H, Hkv, hd, K, lens):
+    """Verify passes of 2 to 132 query vectors per KV head (the tcgen05 attention kernel's
+    four, two and one copies of the vectors and a second row block; every head size), with
+    contexts around a tile of 128 keys, in one tile and in many (clusters of one to eight
+    CTAs, some without keys): logits against the oracle at the step tests' tolerance.  The
+    prompts' prefill runs row blocks of up to 128 vectors."""
+    from paper_2608_10362_gb300 import Engine, _lib
+    from seeded_inputs import ModelShape
+    t = ModelShape(1, 256, H, Hkv, hd, 256, 512)
+    wt = gen_weights(t, 3)
+    oracle = LlamaOracle(t, wt, keep_f64=True)
+    B, S = len(lens), max(lens) + 32
+    eng = Engine(t, wt, max_batch=B, max_seq=S, max_k=K, max_drafts=0, use_graphs=False)
+    try:
+        prompts = [gen_prompt(60 + b, n, t.vocab) for b, n in enumerate(lens)]
+        for b, p in enumerate(prompts):
+            eng.prefill(b, p, seed=b)
+        x = np.stack([gen_prompt(90 + b, K, t.vocab) for b in range(B)]).astype(np.int32)
+        eng.set_batch(B)
+        eng.write_buffer(_lib.BUF_DRAFT_TOKENS, x)
+        eng.verify_step(K)
+        assert eng.sync() == 0
+        z = eng.target_logits(B, K)
+        for b, p in enumerate(prompts):
+            ref = oracle.forward(oracle.new_cache(S), np.concatenate([p, x[b]]))[-(K + 1):]
+            assert np.abs(z[b] - ref).max() <= 1e-3 * np.abs(ref).max()
+    finally:
+        eng.close()
