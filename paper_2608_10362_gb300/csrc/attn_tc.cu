@@ -24,16 +24,21 @@
 // distributed shared memory, each CTA finishing a share of the vectors; sums run in
 // ascending order of warpgroup, copy and CTA.
 //
-// Measured (GB300; us per launch in its pass, before / now): 8B target, 16 requests x 9
-// rows, 512..4096 keys 101 / 50 (a tile of 128 keys takes 1.6, 2560 cycles of it MMAs;
-// 152 SMs' share of HBM allows 1.5; the longest request's CTAs set the time); 7B target,
-// 128 prefill rows at up to 2048 keys 72 / 28; 7B, 5 rows at 2048 keys 15.5 / 13.5.
-// Passes: 8B verify 7.15 / 5.78 ms, 7B verify 2.71 / 2.69, 160M draft of 4 tokens 1.27 /
-// 1.20, 2047 prompt tokens of the 7B 83.8 / 68.5.
+// Measured (GB300; us per launch in its pass, the mma.sync kernel / now): 8B target, 16
+// requests x 9 rows, 512..4096 keys 101 / 45 (a tile of 128 keys takes 1.55, 2560 cycles
+// of it MMAs, 152 SMs' share of HBM allows 1.5; the longest request's CTAs set the
+// time); 7B target, 256 prefill rows at up to 2048 keys 26 (128 rows: 72 / 24); 7B, 5
+// rows at 2048 keys 15.5 / 11.5.  Passes: 8B verify 7.15 / 5.63 ms, 7B verify 2.71 /
+// 2.66, 1.1B verify of 6 rows 0.820 / 0.804, 160M draft of 4 tokens 1.27 / 1.205.
+// Code that each launch fetches anew costs as much as it computes: with 128 keys
+// unrolled and no dry run a prefill launch took 39, a first tile alone 10.
 // Tried instead: the planes of P in the two copies' rows, which saves half of P V's MMAs
-// but gives every thread 128 keys: 0.34 ms more for the 8B verify.
+// but gives every thread 128 keys: 0.34 ms more for the 8B verify; P V of two tiles and
+// then S of two (8B verify 5.85 ms).
 //
-// Roles (320 threads): warps 0-3, 4-7 softmax, 8 copies, 9 MMAs.  K and V tiles pass
+// Roles (384 threads): warps 0-3, 4-7 softmax, 8 copies, 9 MMAs of S, 11 of P V; warp 10 runs the softmax
+// code and the reduction once, dry (no store, no barrier), while the others wait for their
+// predecessor and the first tiles: code that each launch fetches anew.  K and V tiles pass
 // through one ring in the order of their use: K0 K1 V0 K2 V1 ...  Every wait is bounded.
 #include <cuda_bf16.h>
 
@@ -46,7 +51,7 @@ namespace memspec {
 
 namespace {
 
-constexpr int kThreads = 320;
+constexpr int kThreads = 384;
 constexpr int kTile = 128;        // keys per tile
 constexpr int kRows = 128;        // MMA rows
 constexpr int kMaxSlots = 8;
@@ -68,9 +73,10 @@ struct Ctl {
   uint64_t s_full[2];    // S of the warpgroup's tile is complete
   uint64_t p_full[2];    // ... its P is written (4 warps)
   uint64_t o_full[2];    // ... its P V is complete
-  uint64_t drain;
+  uint64_t drain[2];
   uint32_t tmem_base;
   int abort_flag;
+  int at[kRows];         // vector -> its offset in q and out, in heads
 };
 
 __device__ __forceinline__ float ex2(float x) {
@@ -103,28 +109,6 @@ __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, float* v) {
       : "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld_x64(uint32_t taddr, float* v) {
-  uint32_t r[64];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {"
-      "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
-      "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-      "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-        "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 // ... and store (tmem_st_wait completes it).
 __device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t* r) {
@@ -176,6 +160,8 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
   return v;
 }
 
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+
 // Index (floats) of features d..d+3 of partial row r: 16-byte chunks rotated by the
 // row, so that 32 threads storing one row each meet no bank conflicts.
 template <int HD>
@@ -189,7 +175,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   constexpr int kNS = C::kSlots;
   constexpr int kVR = KG;                 // vectors per copy (rows of the copy)
   constexpr int kCopies = kRows / kVR;
-  constexpr int kHold = KG == 64 ? 64 : 32;   // score columns a thread holds at a time
   constexpr uint32_t kO = 256;            // TMEM: S of the two warpgroups, then their O
   constexpr uint32_t kTmemCols = 512;
   __shared__ Ctl ctl;
@@ -216,7 +201,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       mbar_init(&ctl.p_full[w], 4);
       mbar_init(&ctl.o_full[w], 1);
     }
-    mbar_init(&ctl.drain, 1);
+    mbar_init(&ctl.drain[0], 1);
+    mbar_init(&ctl.drain[1], 1);
     ctl.abort_flag = 0;
     fence_mbar_init();
   }
@@ -233,6 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
+  const bool dry = warp == 10, soft = warp < 8 || dry;
 
   const bool early = a.ctx_early != 0;
   if (!early) pdl_wait();
@@ -266,8 +253,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const int row0 = (req * a.Hkv + kvh) * a.max_seq + k0;
       const int loads = 2 * n;
       // load i: K0, then K(t + 1) and V(t) in turn, last V(n - 1)
-      auto tile_of = [&](int i) { return i == 0 ? 0 : (i == loads - 1 ? n - 1 : ((i & 1) ? (i + 1) >> 1 : (i >> 1) - 1)); };
-      auto is_v = [&](int i) { return i > 0 && (i == loads - 1 || (i & 1) == 0); };
+      auto is_v = [&](int i) { return i == loads - 1 || (i > 0 && (i & 1) == 0); };
+      auto tile_of = [&](int i) { return i == loads - 1 ? n - 1 : is_v(i) ? i / 2 - 1 : (i + 1) / 2; };
       auto load = [&](int i, int s) {
         mbar_arrive_expect_tx(&ctl.full[s], C::kSlotBytes);
         tma_load_3d(ring + s * C::kSlotBytes, is_v(i) ? &a.vmap : &a.kmap, 0, row0 + tile_of(i) * kTile, 0,
@@ -294,94 +281,114 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         for (int j = max(0, i - kNS); j < i; ++j) mbar_wait_drain(&ctl.full[j % kNS], static_cast<uint32_t>(j / kNS) & 1u);
     }
     __syncwarp();
-  } else if (warp == 9) {
-    // ------------------------------------------------ MMAs (the warp stays converged; one lane issues)
+  } else if (warp == 9 || warp == 11) {
+    // ------------------------------------------------ MMAs: warp 9 S, warp 11 P V.  The warps
+    // stay converged, one lane issues.  A tcgen05 fence after a wait holds a thread until
+    // its own earlier MMAs have completed (470 cycles of a drained pipe, measured): hence two
+    // threads, and none after the waits for copies, which need none
     const bool lead = elect_one();
-    constexpr uint32_t kIdS = make_idesc_bf16_f32(kRows, kTile);
-    constexpr uint32_t kIdO = make_idesc_bf16_f32(kRows, HD) | (1u << 16);   // B N-major
-    const uint64_t qdesc = make_smem_desc_sw128(smem_addr(qs));
-    const uint64_t kdesc0 = make_smem_desc_sw128(smem_addr(ring));
-    // V tile, N-major: 64-feature columns kTile x 128 bytes apart, 8-key groups 1024
-    const uint64_t vdesc0 = (kdesc0 & ~(0xFFFFull << 16)) | (static_cast<uint64_t>((kTile * 128) >> 4) << 16);
     bool ok = n > 0;
     auto wait = [&](uint64_t* bar, int phase) {
-      ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, static_cast<uint32_t>(phase) & 1u, abort_flag, a.status));
-      tc_fence_after();
+      ok = ok && __all_sync(0xffffffffu, mbar_wait_bounded(bar, static_cast<uint32_t>(phase) & 1u, abort_flag, a.status));
       return ok;
     };
-    int i = 0;   // load consumed next
-    auto mma_s = [&](int t) {
-      const int s = i % kNS;
-      if (!wait(&ctl.full[s], i / kNS)) return;
-      if (lead) {
-        const uint64_t kd = kdesc0 + static_cast<uint32_t>(s * (C::kSlotBytes >> 4));
-        const uint32_t d = tmem + static_cast<uint32_t>((t & 1) * 128);
+    if (warp == 9) {
+      constexpr uint32_t kIdS = make_idesc_bf16_f32(kRows, kTile);
+      const uint64_t qdesc = make_smem_desc_sw128(smem_addr(qs));
+      const uint64_t kdesc0 = make_smem_desc_sw128(smem_addr(ring));
+      wait(&ctl.q_full, 0);
+      for (int t = 0; t < n && ok; ++t) {
+        const int i = t == 0 ? 0 : 2 * t - 1, s = i % kNS;   // load of K(t)
+        if (t >= 2) {   // P of tile t - 2 lies where S of tile t goes
+          if (!wait(&ctl.o_full[t & 1], (t - 2) >> 1)) break;
+          tc_fence_after();
+        }
+        if (!wait(&ctl.full[s], i / kNS)) break;
+        if (lead) {
+          const uint64_t kd = kdesc0 + static_cast<uint32_t>(s * (C::kSlotBytes >> 4));
+          const uint32_t d = tmem + static_cast<uint32_t>((t & 1) * 128);
 #pragma unroll
-        for (int pl = kQPlanes - 1; pl >= 0; --pl)   // small terms first: fewer roundings at full size
+          for (int pl = kQPlanes - 1; pl >= 0; --pl)   // small terms first: fewer roundings at full size
 #pragma unroll
-          for (int ks = 0; ks < HD / 16; ++ks) {
-            const uint32_t off = static_cast<uint32_t>(((ks >> 2) * kTile * 128 + (ks & 3) * 32) >> 4);
-            tc_mma_bf16(d, qdesc + pl * (C::kPlaneBytes >> 4) + off, kd + off, kIdS, pl < kQPlanes - 1 || ks > 0 ? 1u : 0u);
-          }
-        tc_commit(&ctl.empty[s]);
-        tc_commit(&ctl.s_full[t & 1]);
+            for (int ks = 0; ks < HD / 16; ++ks) {
+              const uint32_t off = static_cast<uint32_t>(((ks >> 2) * kTile * 128 + (ks & 3) * 32) >> 4);
+              tc_mma_bf16(d, qdesc + pl * (C::kPlaneBytes >> 4) + off, kd + off, kIdS,
+                          pl < kQPlanes - 1 || ks > 0 ? 1u : 0u);
+            }
+          tc_commit(&ctl.empty[s]);
+          tc_commit(&ctl.s_full[t & 1]);
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      ++i;
-    };
-    if (ok && wait(&ctl.q_full, 0)) mma_s(0);
-    for (int t = 0; t < n && ok; ++t) {
-      if (t + 1 < n) {
-        // P of tile t - 1 lies where S of tile t + 1 goes
-        if (t >= 1 && !wait(&ctl.o_full[(t + 1) & 1], (t - 1) >> 1)) break;
-        mma_s(t + 1);
-        if (!ok) break;
-      }
-      if (!wait(&ctl.p_full[t & 1], t >> 1)) break;
-      const int s = i % kNS;
-      if (!wait(&ctl.full[s], i / kNS)) break;
-      if (lead) {
-        const uint64_t vd = vdesc0 + static_cast<uint32_t>(s * (C::kSlotBytes >> 4));
-        const uint32_t d = tmem + kO + static_cast<uint32_t>((t & 1) * HD);
-        const uint32_t p = tmem + static_cast<uint32_t>((t & 1) * 128);
+    } else {
+      constexpr uint32_t kIdO = make_idesc_bf16_f32(kRows, HD) | (1u << 16);   // B N-major
+      // V tile, N-major: 64-feature columns kTile x 128 bytes apart, 8-key groups 1024
+      const uint64_t vdesc0 = (make_smem_desc_sw128(smem_addr(ring)) & ~(0xFFFFull << 16)) |
+                              (static_cast<uint64_t>((kTile * 128) >> 4) << 16);
+      for (int t = 0; t < n && ok; ++t) {
+        const int i = t == n - 1 ? 2 * n - 1 : 2 * t + 2, s = i % kNS;   // load of V(t)
+        if (!wait(&ctl.full[s], i / kNS) || !wait(&ctl.p_full[t & 1], t >> 1)) break;
+        tc_fence_after();
+        if (lead) {
+          const uint64_t vd = vdesc0 + static_cast<uint32_t>(s * (C::kSlotBytes >> 4));
+          const uint32_t d = tmem + kO + static_cast<uint32_t>((t & 1) * HD);
+          const uint32_t p = tmem + static_cast<uint32_t>((t & 1) * 128);
 #pragma unroll
-        for (int pl = 0; pl < 2; ++pl)
+          for (int pl = 0; pl < 2; ++pl)
 #pragma unroll
-          for (int ks = 0; ks < kTile / 16; ++ks)
-            mma_ts(d, p + (ks >> 1) * 32 + pl * 16 + (ks & 1) * 8, vd + static_cast<uint32_t>((ks * 2048) >> 4), kIdO,
-                   t >= 2 || pl + ks > 0 ? 1u : 0u);
-        tc_commit(&ctl.empty[s]);
-        tc_commit(&ctl.o_full[t & 1]);
+            for (int ks = 0; ks < kTile / 16; ++ks)
+              mma_ts(d, p + (ks >> 1) * 32 + pl * 16 + (ks & 1) * 8, vd + static_cast<uint32_t>((ks * 2048) >> 4), kIdO,
+                     t >= 2 || pl + ks > 0 ? 1u : 0u);
+          tc_commit(&ctl.empty[s]);
+          tc_commit(&ctl.o_full[t & 1]);
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      ++i;
     }
     if (!ok && n > 0 && lead) {   // every MMA issued completes before the CTA leaves
-      tc_commit(&ctl.drain);
-      mbar_wait_drain(&ctl.drain, 0);
+      uint64_t* drain = &ctl.drain[warp == 9 ? 0 : 1];
+      tc_commit(drain);
+      mbar_wait_drain(drain, 0);
     }
     __syncwarp();
   } else {
     // ------------------------------------------------ softmax
-    const int w = warp >> 2;
+    const int w = dry ? 0 : warp >> 2;
     const int row = (warp & 3) * 32 + lane;            // MMA row = TMEM lane
     const int copy = row / kVR, v = row % kVR;         // (copy: the same in the whole warp)
-    if (early) pdl_wait();
+    const int rr = v < nq ? v % nr : 0;
+    if (w == 0 && copy == 0 && !dry && v < nq) ctl.at[v] = (g * R + r_lo + rr) * a.H + kvh * gs + v / nr;
+    if (!dry) named_bar_sync(1, 256);
+    if (early && !dry) pdl_wait();
     if (threadIdx.x == 0) trace_at(trace, 2);
-    if (n > 0) {
+    if (n > 0 && !dry) {
       // Q, scaled, in its planes, K-major with the 128-byte swizzle; every copy.  Rows
-      // without a vector keep what the memory holds: no other row's result sees them
-      for (int idx = threadIdx.x; idx < nq * (HD / 8); idx += 256) {
+      // without a vector keep what the memory holds: no other row's result sees them.
+      // Eight features are 32 bytes of q and 16 of each plane: they land where planes 1
+      // and 2 of them go, all of the CTA's in one round trip
+      const int items = nq * (HD / 8);
+      auto slot = [&](int vv, int ch) { return qs + (ch >> 3) * (kRows * 128) + vv * 128 + (((ch ^ vv) & 7) << 4); };
+#pragma unroll 2
+      for (int idx = threadIdx.x; idx < items; idx += 256) {
         const int vv = idx / (HD / 8), ch = idx % (HD / 8);
-        const int hl = vv / nr, rr = vv - hl * nr;
-        const float4* src = reinterpret_cast<const float4*>(
-            a.q + (static_cast<size_t>(g * R + r_lo + rr) * a.H + kvh * gs + hl) * HD + ch * 8);
-        const float4 x0 = src[0], x1 = src[1];
-        const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        const float* src = a.q + static_cast<size_t>(ctl.at[vv]) * HD + ch * 8;
+        const uint32_t dst = smem_addr(slot(vv, ch)) + C::kPlaneBytes;
+        asm volatile("cp.async.cg.shared.global [%0], [%2], 16;\n\tcp.async.cg.shared.global [%1], [%3], 16;" ::"r"(dst),
+                     "r"(dst + C::kPlaneBytes), "l"(src), "l"(src + 4)
+                     : "memory");
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 1
+      for (int idx = threadIdx.x; idx < items; idx += 256) {
+        const int vv = idx / (HD / 8), ch = idx % (HD / 8);
+        uint8_t* at = slot(vv, ch);
+        const float4 x0 = *reinterpret_cast<const float4*>(at + C::kPlaneBytes);
+        const float4 x1 = *reinterpret_cast<const float4*>(at + 2 * C::kPlaneBytes);
+        const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
         uint32_t pq[kQPlanes][4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          float y0 = x[2 * e] * a.scale_log2, y1 = x[2 * e + 1] * a.scale_log2;
+          float y0 = xs[2 * e] * a.scale_log2, y1 = xs[2 * e + 1] * a.scale_log2;
 #pragma unroll
           for (int pl = 0; pl < kQPlanes; ++pl) {
             pq[pl][e] = bf16x2(y0, y1);
@@ -391,18 +398,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           }
         }
 #pragma unroll
-        for (int c = 0; c < kCopies; ++c) {
-          const int r = c * kVR + vv;
-          uint8_t* dst = qs + (ch >> 3) * (kRows * 128) + r * 128 + (((ch ^ r) & 7) << 4);
+        for (int c = 0; c < kCopies; ++c)   // (a copy's rows are a multiple of the swizzle's eight apart)
 #pragma unroll
           for (int pl = 0; pl < kQPlanes; ++pl)
-            *reinterpret_cast<uint4*>(dst + pl * C::kPlaneBytes) = make_uint4(pq[pl][0], pq[pl][1], pq[pl][2], pq[pl][3]);
-        }
+            *reinterpret_cast<uint4*>(at + c * kVR * 128 + pl * C::kPlaneBytes) =
+                make_uint4(pq[pl][0], pq[pl][1], pq[pl][2], pq[pl][3]);
       }
       fence_proxy_async_smem();
       mbar_arrive(&ctl.q_full);
     }
-    const int rr = v < nq ? v % nr : 0;
     const int p_row = v < nq ? pos0 + r_lo + rr : -1;              // last key the row sees
     const uint32_t amask = tree && v < nq && r_lo + rr < kTreeRows ? plan->anc[r_lo + rr] : 0u;
     const uint32_t lanes = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -410,39 +414,38 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     const uint32_t o_at = tmem + lanes + kO + static_cast<uint32_t>(w * HD);
     float m = -INFINITY, l = 0.f;
     bool ok = true;
-    for (int t = w; t < n; t += 2) {
-      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.s_full[w], static_cast<uint32_t>(t >> 1) & 1u, abort_flag, a.status));
+    for (int t = w; t < (dry ? 1 : n); t += 2) {
+      ok = dry || __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.s_full[w], static_cast<uint32_t>(t >> 1) & 1u, abort_flag, a.status));
       if (!ok) break;
       tc_fence_after();
       if (t == 0 && threadIdx.x == 0) trace_at(trace, 10);
       const int kt0 = k0 + t * kTile;
       const int key0 = kt0 + copy * KG;
-      const bool part = key0 + KG > min(pos0, k1);   // holds keys that some row does not see
+      const bool part = dry || key0 + KG > min(pos0, k1);   // holds keys that some row does not see
       const int lim = min(p_row, k1 - 1);
-      auto mask = [&](float* x, int key1, auto cnt) {
+      auto mask = [&](float* x, int key1) {
         if (!part) return;
+        if (!tree) {
 #pragma unroll
-        for (int e = 0; e < decltype(cnt)::value; ++e) {
-          bool vis = key1 + e <= lim;
-          if (tree) {
-            const int rel = key1 + e - pos0;
-            vis = vis && (rel < 0 || (rel < kTreeRows && ((amask >> rel) & 1u) != 0u));
-          }
+          for (int e = 0; e < 32; ++e) x[e] = key1 + e <= lim ? x[e] : -INFINITY;
+          return;
+        }
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          const int rel = key1 + e - pos0;
+          const bool vis = key1 + e <= lim && (rel < 0 || (rel < kTreeRows && ((amask >> rel) & 1u) != 0u));
           x[e] = vis ? x[e] : -INFINITY;
         }
       };
-      // up to 64 columns stay in registers, 128 are read again for P
-      float s[kHold];
+      // 32 columns at a time; more than 32 are read again for P
+      float s[32];
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+      for (int c = 0; c < KG; c += 32) {
+        tmem_ld_x32(s_at + copy * KG + c, s);
+        mask(s, key0 + c);
 #pragma unroll
-      for (int c = 0; c < KG / kHold; ++c) {
-        if constexpr (kHold == 64)
-          tmem_ld_x64(s_at + copy * KG, s);
-        else
-          tmem_ld_x32(s_at + copy * KG + c * 32, s);
-        mask(s, key0 + c * kHold, std::integral_constant<int, kHold>{});
-#pragma unroll
-        for (int e = 0; e < kHold; ++e) mx[e & 3] = fmaxf(mx[e & 3], s[e]);
+        for (int e = 0; e < 32; ++e) mx[e & 3] = fmaxf(mx[e & 3], s[e]);
       }
       const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
       if (t < 2) {
@@ -453,7 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           const float f = up ? ex2(m - mt) : 1.f;   // m = -inf: 0
           m = up ? mt : m;
           l *= f;
-#pragma unroll
+#pragma unroll 1
           for (int c = 0; c < HD / 32; ++c) {
             float o[32];
             uint32_t u[32];
@@ -468,24 +471,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       float sum[4] = {0.f, 0.f, 0.f, 0.f};
       // P over S, 32 keys in the columns of their scores: 16 columns of the hi plane,
       // 16 of the lo plane, two keys a column
-#pragma unroll
-      for (int c = 0; c < KG / 32; ++c) {
-        if constexpr (kHold < KG) {
-          tmem_ld_x32(s_at + c * 32, s);
-          mask(s, key0 + c * 32, std::integral_constant<int, 32>{});
+#pragma unroll 1
+      for (int c = 0; c < KG; c += 32) {
+        if constexpr (KG > 32) {
+          tmem_ld_x32(s_at + copy * KG + c, s);
+          mask(s, key0 + c);
         }
-        const float* sc = s + (kHold < KG ? 0 : c * 32);
         uint32_t p[32];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-          const float p0 = ex2(sc[2 * e] - mu), p1 = ex2(sc[2 * e + 1] - mu);
+          const float p0 = ex2(s[2 * e] - mu), p1 = ex2(s[2 * e + 1] - mu);
           sum[(2 * e) & 3] += p0;
           sum[(2 * e + 1) & 3] += p1;
           p[e] = bf16x2(p0, p1);
           const float2 h = unpack2(p[e]);
           p[16 + e] = bf16x2(p0 - h.x, p1 - h.y);
         }
-        tmem_st_x32(s_at + copy * KG + c * 32, p);
+        if (!dry) tmem_st_x32(s_at + copy * KG + c, p);
       }
       l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
       if constexpr (kCopies > 1) {   // zeros for the other copies' keys
@@ -494,10 +496,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         for (int e = 0; e < 32; ++e) z[e] = 0u;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          if (c / (KG / 32) != copy) tmem_st_x32(s_at + c * 32, z);
+          if (c / (KG / 32) != copy && !dry) tmem_st_x32(s_at + c * 32, z);
       }
       tmem_st_wait();
-      if (kt0 + kTile > k1) {   // V rows past the last key hold anything: zeros
+      if (kt0 + kTile > k1 && !dry) {   // V rows past the last key hold anything: zeros
         const int i = 2 * n - 1;
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.full[i % kNS], static_cast<uint32_t>(i / kNS) & 1u, abort_flag, a.status));
         if (!ok) break;
@@ -511,20 +513,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl.p_full[w]);
+      if (lane == 0 && !dry) mbar_arrive(&ctl.p_full[w]);
     }
     const int mine = (n - w + 1) >> 1;   // tiles of this warpgroup
-    if (ok && mine > 0)
+    if (ok && mine > 0 && !dry)
       ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl.o_full[w], static_cast<uint32_t>(mine - 1) & 1u, abort_flag, a.status));
     tc_fence_after();
     if (threadIdx.x == 0) trace_at(trace, 9);
     // the CTA's partial rows: weights against the vector's max, then the sum
     if (n > 0) {
       float* red = reinterpret_cast<float*>(ring);
-      named_bar_sync(1, 256);   // every MMA of the CTA has completed: the ring and Q are free
-      ml[w * kRows + row] = make_float2(m, l);
-      named_bar_sync(1, 256);
-      ok = ok && !*abort_flag;
+      if (!dry) {
+        named_bar_sync(1, 256);   // every MMA of the CTA has completed: the ring and Q are free
+        ml[w * kRows + row] = make_float2(m, l);
+        named_bar_sync(1, 256);
+      }
       float M = -INFINITY, L = 0.f;
 #pragma unroll
       for (int q = 0; q < 2 * kCopies; ++q) M = fmaxf(M, ml[q / kCopies * kRows + (q % kCopies) * kVR + v].x);
@@ -533,13 +536,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const float2 x = ml[q / kCopies * kRows + (q % kCopies) * kVR + v];
         if (x.x != -INFINITY) L += ex2(x.x - M) * x.y;
       }
-      if (w == 0 && copy == 0) cml[v] = make_float2(M, L);
+      if (w == 0 && copy == 0 && !dry) cml[v] = make_float2(M, n_cta == 1 ? 1.f / L : L);
       const float f = m == -INFINITY ? 0.f : ex2(m - M);
-#pragma unroll
+#pragma unroll 1
       for (int c = 0; c < HD / 32; ++c) {
         float o[32];
         tmem_ld_x32(o_at + c * 32, o);
-        if (v < nq) {
+        if (v < nq && !dry) {
 #pragma unroll
           for (int e = 0; e < 32; e += 4) {
             const bool z = m == -INFINITY;   // no visible key, or no tile: O holds anything
@@ -555,23 +558,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 
   // every CTA of the cluster: reduce its own rows, then finish a share of the vectors
   float* red = reinterpret_cast<float*>(ring);
-  const bool soft = warp < 8;
   constexpr int kV4 = HD / 4;
-  auto emit = [&](int vv, int d, float4 o, float L) {
-    const float li = 1.f / L;
-    const int hl = vv / nr, rr = vv - hl * nr;
-    const size_t oi = (static_cast<size_t>(g * R + r_lo + rr) * a.H + kvh * gs + hl) * HD + d;
+  const int tid = dry ? lane : static_cast<int>(threadIdx.x);
+  auto emit = [&](int vv, int d, float4 o, float li) {   // li: 1 / sum
+    const size_t oi = static_cast<size_t>(ctl.at[vv]) * HD + d;
     const float y[4] = {o.x * li, o.y * li, o.z * li, o.w * li};
     __nv_bfloat16 hv[4], lv[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) split_bf16(y[e], hv[e], lv[e]);
+    if (dry) return;
     *reinterpret_cast<uint2*>(a.out + oi) = *reinterpret_cast<const uint2*>(hv);
     if (a.out_lo != nullptr) *reinterpret_cast<uint2*>(a.out_lo + oi) = *reinterpret_cast<const uint2*>(lv);
   };
   if (soft && n > 0) {
-    named_bar_sync(1, 256);
+    if (!dry) named_bar_sync(1, 256);
     const bool good = !*abort_flag;
-    for (int idx = threadIdx.x; idx < nq * kV4 && good; idx += 256) {
+#pragma unroll 2
+    for (int idx = tid; idx < (!good ? 0 : dry ? kV4 : nq * kV4); idx += 256) {
       const int vv = idx / kV4, d = (idx % kV4) * 4;
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -584,46 +587,72 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       if (n_cta == 1)
         emit(vv, d, o, cml[vv].y);
-      else
+      else if (!dry)
         *reinterpret_cast<float4*>(red + red_at<HD>(vv, d)) = o;   // this thread alone reads that place
     }
   }
   if (n_cta > 1) {
-    cluster_arrive_release();
-    cluster_wait_acquire();
-    if (threadIdx.x == 0) trace_at(trace, 6);
-    if (soft && work && !*abort_flag) {
-      const uint32_t red_addr = smem_addr(red), cml_addr = smem_addr(cml);
-      const int lo = nq * split / n_cta, hi = nq * (split + 1) / n_cta;
-      for (int idx = lo * kV4 + threadIdx.x; idx < hi * kV4; idx += 256) {
-        const int vv = idx / kV4, d = (idx % kV4) * 4;
-        float2 st[8];
-        float4 x[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < n_active) {
-            st[q] = ld_cluster_f2(mapa_shared(cml_addr + vv * 8, q));
-            x[q] = ld_cluster_f4(mapa_shared(red_addr + red_at<HD>(vv, d) * 4, q));
-          }
-        float M = -INFINITY, L = 0.f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < n_active) M = fmaxf(M, st[q].x);
-        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < n_active) {
-            const float f = st[q].x == -INFINITY ? 0.f : ex2(st[q].x - M);
-            L += f * st[q].y;
-            o.x += f * x[q].x;
-            o.y += f * x[q].y;
-            o.z += f * x[q].z;
-            o.w += f * x[q].w;
-          }
-        emit(vv, d, o, L);
-      }
+    if (!dry) {
+      cluster_arrive_release();
+      cluster_wait_acquire();
     }
-    cluster_arrive_release();   // no CTA leaves while another reads its rows
+    if (threadIdx.x == 0) trace_at(trace, 6);
+    if (soft && work) {
+      const uint32_t red_addr = smem_addr(red), cml_addr = smem_addr(cml);
+      const int lo = nq * split / n_cta, hi = dry ? lo + 1 : nq * (split + 1) / n_cta;
+      const int n_src = dry ? 1 : n_active, src0 = dry ? split : 0;   // (dry: this CTA's own memory)
+      // kB x four features of this CTA's vectors from kQ CTAs in one round trip
+      auto combine = [&](auto q_c, auto b_c) {
+        constexpr int kQ = decltype(q_c)::value, kB = decltype(b_c)::value;
+        for (int base = lo * kV4 + tid; base < hi * kV4; base += 256 * kB) {
+          float2 st[kB][kQ];
+          float4 x[kB][kQ];
+#pragma unroll
+          for (int b = 0; b < kB; ++b) {
+            const int idx = min(base + b * 256, hi * kV4 - 1);
+            const int vv = idx / kV4, at = red_at<HD>(vv, (idx % kV4) * 4) * 4;
+#pragma unroll
+            for (int q = 0; q < kQ; ++q)
+              if (q < n_src) {
+                st[b][q] = ld_cluster_f2(mapa_shared(cml_addr + vv * 8, src0 + q));
+                x[b][q] = ld_cluster_f4(mapa_shared(red_addr + at, src0 + q));
+              }
+          }
+#pragma unroll
+          for (int b = 0; b < kB; ++b) {
+            const int idx = base + b * 256;
+            if (idx >= hi * kV4) break;
+            float M = -INFINITY, L = 0.f;
+#pragma unroll
+            for (int q = 0; q < kQ; ++q)
+              if (q < n_src) M = fmaxf(M, st[b][q].x);
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < kQ; ++q)
+              if (q < n_src) {
+                const float f = st[b][q].x == -INFINITY ? 0.f : ex2(st[b][q].x - M);
+                L += f * st[b][q].y;
+                o.x += f * x[b][q].x;
+                o.y += f * x[b][q].y;
+                o.z += f * x[b][q].z;
+                o.w += f * x[b][q].w;
+              }
+            emit(idx / kV4, (idx % kV4) * 4, o, 1.f / L);
+          }
+        }
+      };
+      if (n_cta == 2)
+        combine(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+      else if (n_cta == 8)
+        combine(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
+      else
+        combine(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
+    }
+    if (dry) {
+      cluster_arrive_release();
+      cluster_wait_acquire();
+    }
+    cluster_arrive_relaxed();   // no CTA leaves while another reads its rows (all were used)
     cluster_wait_acquire();
   }
   __syncthreads();
