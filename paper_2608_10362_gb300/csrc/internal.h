@@ -14,7 +14,7 @@ typedef __nv_bfloat16 bf16;
 
 constexpr int kMaxGroups = 64;      // requests stepped together
 constexpr int kMaxRows = 256;       // rows of one forward pass (MMA N <= 256)
-constexpr int kPrefillChunk = 128;  // rows per prefill forward
+constexpr int kPrefillChunk = 256;  // rows per prefill forward, at most
 constexpr int kSmallRows = 8;       // rows (two planes) of a pass that runs gemm_small.cu
 constexpr int kMaxK = 15;           // largest draft length
 constexpr int kMaxDrafts = 16;
