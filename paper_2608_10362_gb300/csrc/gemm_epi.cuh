@@ -373,6 +373,8 @@ __device__ __forceinline__ void reduce_partials(const GemmArgs& a, int rt, int c
   const int KT = a.k_tiles;
   const int chunks = (a.rows_total + 15) / 16;
   const int unit = a.pairs ? rt >> 1 : rt;       // tile of the stream-K order
+  // the contributor whose range the tile starts in: its last tile, unless it starts there
+  const int sl_first = sk_begin(c_first, T, G) >= unit * KT ? 0 : 1;
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = 0.f;
   for (int cc0 = c_first; cc0 <= c_last; cc0 += N) {
@@ -381,7 +383,7 @@ __device__ __forceinline__ void reduce_partials(const GemmArgs& a, int rt, int c
     for (int q = 0; q < N; ++q) {
       const int cc = cc0 + q;
       if (cc <= c_last) {
-        const int sl = (sk_begin(cc, T, G) >= unit * KT) ? 0 : 1;
+        const int sl = cc > c_first ? 0 : sl_first;
         const int slot = a.pairs ? pair_slot(a, unit, cc, rt & 1, sl) : 2 * cc + sl;
         const float* pp = a.partials + part_offset(slot, chunks, chunk, et);
 #pragma unroll
