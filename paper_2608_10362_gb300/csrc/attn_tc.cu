@@ -34,7 +34,11 @@
 // unrolled and no dry run a prefill launch took 39, a first tile alone 10.
 // Tried instead: the planes of P in the two copies' rows, which saves half of P V's MMAs
 // but gives every thread 128 keys: 0.34 ms more for the 8B verify; P V of two tiles and
-// then S of two (8B verify 5.85 ms).
+// then S of two (8B verify 5.85 ms); the tiles of all units dealt to one CTA per SM in
+// equal runs, units in several CTAs finished by the last to arrive: 8B at 512..4096 keys
+// 1.551 -> 1.548 ms in 8 layers, but at 16 x 3000 keys 1.513 -> 1.572 (a segment costs 5
+// us besides its tiles), parts of units as CTAs of their own in order of size 1.573 ->
+// 1.604.
 //
 // Roles (384 threads): warps 0-3, 4-7 softmax, 8 copies, 9 MMAs of S, 11 of P V; warp 10 runs the softmax
 // code and the reduction once, dry (no store, no barrier), while the others wait for their
@@ -276,9 +280,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         }
         load(i, s);
       }
-      // after a wait that ran out: leave no copy in flight
-      if (!ok)
-        for (int j = max(0, i - kNS); j < i; ++j) mbar_wait_drain(&ctl.full[j % kNS], static_cast<uint32_t>(j / kNS) & 1u);
+      // the CTA leaves when the last MMAs have signalled their slots; after a wait that ran
+      // out, when no copy is in flight
+      for (int j = max(0, i - kNS); j < i; ++j)
+        mbar_wait_drain(ok ? &ctl.empty[j % kNS] : &ctl.full[j % kNS], static_cast<uint32_t>(j / kNS) & 1u);
     }
     __syncwarp();
   } else if (warp == 9 || warp == 11) {

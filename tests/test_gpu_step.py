@@ -217,14 +217,19 @@ def test_verify_pass_row_counts(B, K):
         eng.close()
 
 
-@pytest.mark.parametrize("H,Hkv,hd,K", [(2, 2, 64, 1), (16, 2, 64, 3), (16, 2, 64, 4), (16, 2, 64, 7), (16, 2, 64, 8),
-                                        (16, 2, 64, 15), (1, 1, 128, 8), (4, 1, 128, 8), (12, 1, 128, 10)])
-@pytest.mark.parametrize("lens", [(3,), (120, 128, 129), (258, 265, 266), (1100, 30)])
+_MANY = [(2, 2, 64, 1), (16, 2, 64, 3), (16, 2, 64, 4), (16, 2, 64, 7), (16, 2, 64, 8), (16, 2, 64, 15), (1, 1, 128, 8),
+         (4, 1, 128, 8), (12, 1, 128, 10)]
+_LENS = [(3,), (120, 128, 129), (258, 265, 266), (1100, 30)]
+_WIDE = [((32, 16, 64, 4), (3, 500, 130, 1000, 64, 257)), ((16, 16, 128, 8), (3, 500, 130, 1000, 64, 257)),
+         ((128, 16, 64, 8), (5, 700, 5, 5, 130, 5)), ((32, 16, 64, 4), (90, 90, 90, 90, 90, 90))]
+
+
+@pytest.mark.parametrize("H,Hkv,hd,K,lens", [(*m, l) for l in _LENS for m in _MANY] + [(*m, l) for m, l in _WIDE])
 def test_attention_of_many_vectors(H, Hkv, hd, K, lens):
     """Verify passes of 2 to 132 query vectors per KV head (the tcgen05 attention kernel's
     four, two and one copies of the vectors and a second row block; every head size), with
     contexts around a tile of 128 keys, in one tile and in many (clusters of one to eight
-    CTAs, some without keys): logits against the oracle at the step tests' tolerance.  The
+    CTAs, some without keys; 96 units: one CTA each): logits against the oracle at the step tests' tolerance.  The
     prompts' prefill runs row blocks of up to 128 vectors, and last passes of 1, 8 and 9
     rows."""
     from paper_2608_10362_gb300 import Engine, _lib
