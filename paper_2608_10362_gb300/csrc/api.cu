@@ -2336,6 +2336,8 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
                                                              align256(static_cast<size_t>(a.row_tiles) * 4));
   a.plan = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // set-up overlaps the previous kernel's end; every read, the weights' too, comes after it
+  a.w_after_wait = 1;
   bool maps;
   cudaError_t e = cudaSuccess;
   if (rows <= 16) {   // gemm_small.cu, rows of one plane
@@ -2345,8 +2347,7 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
     maps = a.x4d ? encode_x4(&a.map_b, x, rows, k, 1, static_cast<long long>(k) * 2, 16, 1) &&
                        encode_x4(&a.map_b2, x, rows, k, 1, static_cast<long long>(k) * 2, 16, gemm_small_x_group())
                  : encode_map(&a.map_b, x, rows, k, 16);
-    a.w_after_wait = 1;
-    if (maps) e = launch_gemm_small(a, grid, st, true);   // set-up overlaps the previous kernel's end
+    if (maps) e = launch_gemm_small(a, grid, st, true);
   } else {
     a.pairs = gemm_pairs(rows, 0, a.row_tiles, a.k_tiles);
     a.n_pad = a.pairs ? gemm_pair_pad(rows, 0) : n_pad;
@@ -2358,8 +2359,8 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
     const int units = a.pairs ? (a.row_tiles + 1) / 2 : a.row_tiles;
     a.split_epi = sk_split_free(units * a.k_tiles, a.k_tiles, grid) ? 0 : 1;
     if (maps)
-      e = a.pairs ? launch_gemm_pair(a, st, false)
-                  : launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages), st, false);
+      e = a.pairs ? launch_gemm_pair(a, st, true)
+                  : launch_gemm(a, grid, gemm_smem_bytes(n_pad, a.stages), st, true);
     if (maps && e == cudaSuccess && a.split_epi) e = launch_gemm_split_epi(a, grid, st, true);
   }
   if (!maps) {

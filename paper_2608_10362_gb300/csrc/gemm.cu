@@ -9,15 +9,9 @@
 //  * swap-AB: the weight tile is the MMA's M=128 operand, the activation rows
 //    are its N (16..256) operand; tcgen05.mma.kind::f16 (bf16 in, fp32 out)
 //    accumulates in TMEM;
-//  * weight tiles [128 rows x 64 k] arrive by TMA (128-byte swizzle) into a
-//    multi-stage mbarrier ring; they are independent of earlier kernels, so the
-//    producer starts streaming before griddepcontrol.wait (programmatic
-//    dependent launch hides the previous kernel's tail);
-//  * activation tiles [n_pad rows x 64 k] arrive by TMA on the same barrier,
-//    issued only after griddepcontrol.wait (they are the previous kernel's
-//    output); RMSNorm is folded in: the previous epilogue wrote bf16(h * gain)
-//    and per-row-tile sums of squares, and this kernel's epilogue scales each
-//    output row by rsqrt(mean(h^2) + eps) (exact: the scale is per row);
+//  * weight tiles [128 rows x 64 k] and activation tiles [n_pad rows x 64 k] arrive
+//    by TMA (128-byte swizzle) into a multi-stage ring, a stage's copies on one
+//    mbarrier, all after griddepcontrol.wait;
 //  * stream-K: the (row-tile, k-tile) space is cut into one contiguous range
 //    per CTA, one CTA per SM; a row tile split over several CTAs is reduced by
 //    the last-arriving CTA in ascending CTA order (deterministic, no float
@@ -51,15 +45,13 @@ struct SmemCtl {
   float red[4][16];
 };
 
-template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_constant__ GemmArgs a) {
   __shared__ SmemCtl ctl;
   extern __shared__ uint8_t dsmem_raw[];
   uint8_t* dsmem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(dsmem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int S = a.stages;
-  const int plane_bytes = a.n_pad * 128;              // one [n_pad][64] bf16 activation plane
-  const int b_bytes = plane_bytes * (a.split ? 2 : 1);
+  const int b_bytes = a.n_pad * 128;                  // [n_pad][64] bf16 activations
   const uint32_t stage_tx = static_cast<uint32_t>(kABytes + b_bytes);
   uint8_t* smem_a = dsmem;
   uint8_t* smem_b = dsmem + static_cast<size_t>(S) * kABytes;
@@ -72,8 +64,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
   const int G = gridDim.x, c = blockIdx.x;
   const int t_begin = sk_begin(c, T, G), t_end = sk_begin(c + 1, T, G);
   const int KT = a.k_tiles;
-  const int layout = !a.split ? kPlain : (2 * a.n_pad <= 256 ? kWide : kTwice);
-  const int acols = acc_cols(a, layout);                 // accumulator columns per buffer
+  const int acols = acc_cols(a, kPlain);                 // accumulator columns per buffer
   const uint32_t tmem_cols = tmem_cols_for(acols);
 
   if (threadIdx.x == 0) {
@@ -108,62 +99,36 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
-    // Weight tiles do not depend on earlier kernels: the first S of them are
-    // requested before griddepcontrol.wait.  Activation tiles are requested after.
+    // The weights' maps point at the caller's matrix, which earlier work on the stream may
+    // write: every copy comes after the wait.
     if (lane == 0) {
-      if (a.a_packed == nullptr) {
-        tma_prefetch_desc(&a.map_a);
-        if (a.pair) tma_prefetch_desc(&a.map_a2);
-      }
+      tma_prefetch_desc(&a.map_a);
       tma_prefetch_desc(&a.map_b);
-      if (a.split) tma_prefetch_desc(&a.map_b2);
-      const uint64_t pol = a.l2_hint == L2_EVICT_FIRST  ? l2_policy_evict_first()
-                           : a.l2_hint == L2_EVICT_LAST ? l2_policy_evict_last()
-                                                        : l2_policy_evict_normal();
+      const uint64_t pol = l2_policy_evict_first();
       const uint64_t pol_b = l2_policy_evict_last();   // activations are re-read by every CTA
       uint32_t issued_mask = 0, last_par = 0;
       bool ok = true;
       const int n_pre = min(S, t_end - t_begin);
       // One thread issues every copy, so the loop is lean: the ring position and
       // the tile coordinates advance incrementally (no division per tile).
-      const uint8_t* wsrc = a.a_packed != nullptr
-                                ? a.a_packed + static_cast<size_t>(t_begin) * kABytes : nullptr;
       int rt = t_begin / KT, kt = t_begin - rt * KT;
       auto load_a = [&](int slot) {
-        uint8_t* dst = smem_a + static_cast<size_t>(slot) * kABytes;
-        if (wsrc != nullptr) {
-          bulk_load(dst, wsrc, kABytes, &ctl.full[slot], pol);
-          wsrc += kABytes;
-        } else if (a.pair) {
-          tma_load_2d(dst, &a.map_a, kt * kTileK, rt * 64, &ctl.full[slot], pol);
-          tma_load_2d(dst + kABytes / 2, &a.map_a2, kt * kTileK, rt * 64, &ctl.full[slot], pol);
-        } else {
-          tma_load_2d(dst, &a.map_a, kt * kTileK, rt * kTileM, &ctl.full[slot], pol);
-        }
+        tma_load_2d(smem_a + static_cast<size_t>(slot) * kABytes, &a.map_a, kt * kTileK, rt * kTileM, &ctl.full[slot], pol);
       };
       auto load_b = [&](int slot, int k_tile) {
-        uint8_t* dst = smem_b + static_cast<size_t>(slot) * b_bytes;
-        tma_load_2d(dst, &a.map_b, k_tile * kTileK, 0, &ctl.full[slot], pol_b);
-        if (a.split) tma_load_2d(dst + plane_bytes, &a.map_b2, k_tile * kTileK, 0, &ctl.full[slot], pol_b);
+        tma_load_2d(smem_b + static_cast<size_t>(slot) * b_bytes, &a.map_b, k_tile * kTileK, 0, &ctl.full[slot], pol_b);
       };
-      // weights of the first n_pre tiles (the ring is empty: no wait needed)
-      const int kt_first = kt;
+      pdl_wait();
+      trace_at(trace, 2);
+      // the first n_pre tiles (the ring is empty: no wait needed)
       for (int p = 0; p < n_pre; ++p) {
         mbar_arrive_expect_tx(&ctl.full[p], stage_tx);
         load_a(p);
+        load_b(p, kt);
         issued_mask |= 1u << p;
         if (++kt == KT) {
           kt = 0;
           ++rt;
-        }
-      }
-      pdl_wait();
-      trace_at(trace, 2);
-      {
-        int k2 = kt_first;
-        for (int p = 0; p < n_pre; ++p) {
-          load_b(p, k2);
-          if (++k2 == KT) k2 = 0;
         }
       }
       int s = n_pre == S ? 0 : n_pre;
@@ -197,13 +162,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
     // The whole warp walks the tiles and one elected lane issues, so that descriptors
     // and loop counters stay in uniform registers.
     const bool lead = elect_one();
-    const uint32_t idesc = make_idesc_bf16_f32(kTileM, layout == kWide ? 2 * a.n_pad : a.n_pad);
+    const uint32_t idesc = make_idesc_bf16_f32(kTileM, a.n_pad);
     // descriptors of stage 0; a stage's (and a k-step's) are offsets in the
     // start-address field (address >> 4, 14 bits: shared memory < 256 KB)
     const uint64_t adesc0 = make_smem_desc_sw128(smem_addr(smem_a));
     const uint64_t bdesc0 = make_smem_desc_sw128(smem_addr(smem_b));
     const uint32_t a_step = kABytes >> 4, b_step = static_cast<uint32_t>(b_bytes) >> 4;
-    const uint32_t p_step = static_cast<uint32_t>(plane_bytes) >> 4;
     int s = 0, seg = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -226,17 +190,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
         const uint32_t acc0 = tt > t ? 1u : 0u;
         if (lead) {
           if (tt == t_begin) trace_at(trace, 3);
-          if (layout != kTwice) {   // one MMA per k-step (N = n_pad or 2 n_pad)
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk)
-              tc_mma_bf16(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-          } else {                  // hi then lo plane into the same accumulator
-#pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk) {
-              tc_mma_bf16(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-              tc_mma_bf16(d_tmem, ad + 2 * kk, bd + p_step + 2 * kk, idesc, 1u);
-            }
-          }
+          for (int kk = 0; kk < kTileK / 16; ++kk)
+            tc_mma_bf16(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
           tc_commit(&ctl.empty[s]);
         }
         __syncwarp();
@@ -259,20 +215,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
     // a warp may only read TMEM lanes 32*(warp % 4) .. +31: that is its feature block
     const int ew = warp & 3;
     const int et = ew * 32 + lane;  // tile feature == TMEM lane
-    // the dry run overlaps the previous launch's tail; the real context follows
-    // (ctx_early: the row plan is final before the wait, so the real context is
-    // built there and the dry run uses it)
-    if (a.ctx_early) {
-      epi_prologue<EPI>(a, ectx, et);
-      if (a.warm) epilogue_warmup<EPI>(a, ectx, ctl.red, stage, rms, c, G, et);
-    } else if (a.warm) {
-      epi_ctx_dry(ectx, a.n_pad, et);
-      epilogue_warmup<EPI>(a, ectx, ctl.red, stage, rms, c, G, et);
-    }
     pdl_wait();
     if (threadIdx.x == 64) trace_at(trace, 13);
-    if (a.rms) rms_prologue(a, rms, et);
-    if (!a.ctx_early) epi_prologue<EPI>(a, ectx, et);
+    epi_prologue<EPI_F32>(a, ectx, et);
     int seg = 0;
     for (int t = t_begin; t < t_end; ++seg) {
       const int rt = t / KT;
@@ -291,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
       named_bar_sync(1, 128);
       if (!ok) break;
       tc_fence_after();
-      epilogue_segment<EPI>(a, ectx, layout, acols, tmem_base, buf, seg, c, G, rt, k0, k1, stage, rms, ctl.red,
+      epilogue_segment<EPI_F32>(a, ectx, kPlain, acols, tmem_base, buf, seg, c, G, rt, k0, k1, stage, rms, ctl.red,
                             &ctl.reduce_flag, ctl.acc_empty, et, ew, lane, threadIdx.x == 64 ? trace : nullptr);
       t = seg_end;
     }
@@ -313,19 +258,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
 // in flight per SM; a budget under ~110 KB lets the next kernel's CTA start on
 // the same SM early (programmatic dependent launch).  MEMSPEC_GEMM_SMEM_KB
 // overrides the default (for measurement).
-static int gemm_budget_bytes(int n_pad) {
+static int gemm_budget_bytes() {
   static int env_kb = -1;
   if (env_kb < 0) {
     const char* e = std::getenv("MEMSPEC_GEMM_SMEM_KB");
     env_kb = e != nullptr ? std::atoi(e) : 0;
   }
   if (env_kb > 0) return env_kb * 1024;
-  return n_pad <= 32 ? 200 * 1024 : 200 * 1024;
+  return 200 * 1024;
 }
 
 int gemm_pick_stages(int n_pad, int planes) {
   const int stage = kABytes + n_pad * 128 * planes;
-  const int budget = gemm_budget_bytes(n_pad);
+  const int budget = gemm_budget_bytes();
   const int fixed = kTileM * kStagePitch * 4 + kMaxRows * 4 + static_cast<int>(sizeof(EpiCtx)) + 1024;
   int s = (budget - fixed) / stage;
   if (s > kMaxStages) s = kMaxStages;
@@ -340,7 +285,7 @@ size_t gemm_smem_bytes(int n_pad, int stages, int planes) {
 
 cudaError_t gemm_set_max_smem() {
   // 227 KB per block minus the kernel's static shared memory
-  return cudaFuncSetAttribute(gemm_stream_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+  return cudaFuncSetAttribute(gemm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
 }
 
 cudaError_t launch_gemm(const GemmArgs& a, int grid, size_t smem, cudaStream_t s, bool pdl) {
@@ -355,7 +300,7 @@ cudaError_t launch_gemm(const GemmArgs& a, int grid, size_t smem, cudaStream_t s
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_stream_kernel<EPI_F32>, a);
+  return cudaLaunchKernelEx(&cfg, gemm_stream_kernel, a);
 }
 
 }  // namespace memspec

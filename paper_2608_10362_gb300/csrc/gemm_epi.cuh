@@ -122,8 +122,7 @@ template <int EPI>
 static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiCtx* ctx,
                                                    float (*red)[16], float* stage,
                                                    const float* rms, int rt, int chunk, int et,
-                                                   const float* vin, unsigned long long* ts,
-                                                   bool dry) {
+                                                   const float* vin, unsigned long long* ts) {
   const int ew = et >> 5, lane = et & 31;
   constexpr int epi = EPI;
   const int rows_total = a.rows_total;
@@ -146,8 +145,8 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
       for (int j = 0; j < 16; ++j) {
         const int r = r0 + j;
         if (last_only) {
-          if (ctx_bit(ctx->last, r) && !dry) out[ctx->grp[r] * gstride + f] = v[j];
-        } else if (ctx_bit(ctx->valid, r) && !dry) {
+          if (ctx_bit(ctx->last, r)) out[ctx->grp[r] * gstride + f] = v[j];
+        } else if (ctx_bit(ctx->valid, r)) {
           out[static_cast<size_t>(r) * out_ld + f] = v[j];
         }
       }
@@ -177,7 +176,7 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const int r = r0 + j;
-      if (r >= rows_total || dry) continue;
+      if (r >= rows_total) continue;
       const size_t o = static_cast<size_t>(r) * h_ld + f;
       h[o] = hn[j];
       if (gain_next != nullptr)
@@ -203,7 +202,7 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
     trace_at(ts, 10);
     if (et < 16) {
       const int r = r0 + et;
-      if (r < rows_total && !dry) {
+      if (r < rows_total) {
         const float s = ((red[0][et] + red[1][et]) + red[2][et]) + red[3][et];
         ss_out[static_cast<size_t>(rt) * ss_stride + r] = s;
       }
@@ -233,7 +232,6 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
             const float g = stage[et * kStagePitch + j];
             const float u = stage[(et + 64) * kStagePitch + j];
             const float y = g / (1.0f + expf(-g)) * u;
-            if (dry) continue;
             const size_t o = static_cast<size_t>(r) * act_ld + f;
             store_split_bf16(act + o, act_lo != nullptr ? act_lo + o : nullptr, y);
           }
@@ -277,7 +275,6 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
             const float x2 = stage[(e1 + half_hd) * kStagePitch + j];
             y = d < half_hd ? (x1 * c - x2 * sn) : (x1 * sn + x2 * c);
           }
-          if (dry) continue;
           if (seg == 0) {
             q_out[static_cast<size_t>(r) * q_dim + f] = y;
           } else {
@@ -306,7 +303,6 @@ static __device__ __noinline__ void apply_epilogue(const GemmArgs& a, const EpiC
             y[j] = d < half_hd ? (x1 * c - x2 * sn) : (x1 * sn + x2 * c);
           }
         }
-        if (dry) ok_mask = 0;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           if (!(ok_mask & (1u << j))) continue;
@@ -405,45 +401,6 @@ __device__ __forceinline__ void reduce_partials(const GemmArgs& a, int rt, int c
   }
 }
 
-// Synthetic context for the dry run (below): every row valid, position and
-// request 0, so every address the dry run forms is in bounds.  Ends with a barrier.
-__device__ __forceinline__ void epi_ctx_dry(EpiCtx* ctx, int n_pad, int et) {
-  for (int r = et; r < n_pad; r += 128) {
-    ctx->pos[r] = 0;
-    if (r < kTreeRows) ctx->rpos[r] = 0;
-    ctx->req[r] = 0;
-    ctx->grp[r] = 0;
-  }
-  if (et < kMaxRows / 32) {
-    ctx->valid[et] = 0xffffffffu;
-    ctx->last[et] = 0u;
-  }
-  for (int i = et; i < kCtxRopeRows * 64; i += 128) {
-    ctx->rc[i / 64][i % 64] = 1.f;
-    ctx->rs[i / 64][i % 64] = 0.f;
-  }
-  named_bar_sync(1, 128);
-}
-
-// Dry run of the tail - the partial reduction and the epilogue of this CTA's
-// first row tile, with every global store off - by the 128 epilogue threads
-// before the launch waits for its predecessor (griddepcontrol.wait): it only
-// reads scratch and weights, with the synthetic context of epi_ctx_dry.  The
-// tail runs once per launch; without this its instructions are fetched cold,
-// one miss after another, on the critical path.
-template <int EPI>
-__device__ __forceinline__ void epilogue_warmup(const GemmArgs& a, const EpiCtx* ctx,
-                                                float (*red)[16], float* stage, const float* rms,
-                                                int c, int G, int et) {
-  const int KT = a.k_tiles, T = a.row_tiles * KT;
-  float v[16];
-  const int rt = sk_begin(c, T, G) / KT;
-  const int c_first = sk_cta_of(rt * KT, T, G);
-  const int c_last = sk_cta_of((rt + 1) * KT - 1, T, G);
-  reduce_partials(a, rt, c_first, c_last, 0, et, T, G, v);
-  apply_epilogue<EPI>(a, ctx, red, stage, rms, rt, 0, et, v, nullptr, true);
-}
-
 // Epilogue of one accumulated segment [k0, k1) of row tile rt, run by the 128
 // epilogue threads (et = TMEM lane = tile feature).  `c` is this CTA's index and
 // G the op's grid; T = row_tiles * k_tiles.  The caller has waited for the
@@ -477,7 +434,7 @@ __device__ __forceinline__ void epilogue_segment(const GemmArgs& a, const EpiCtx
   if (full) {
     for (int chunk = 0; chunk < a.n_pad / 16; ++chunk) {
       load_chunk(chunk);
-      apply_epilogue<EPI>(a, ctx, red, stage, rms, rt, chunk, et, v, nullptr, false);
+      apply_epilogue<EPI>(a, ctx, red, stage, rms, rt, chunk, et, v, nullptr);
     }
   } else {
     for (int chunk = 0; chunk < a.n_pad / 16; ++chunk) {
@@ -510,7 +467,7 @@ __device__ __forceinline__ void epilogue_segment(const GemmArgs& a, const EpiCtx
   for (int chunk = 0; chunk < a.n_pad / 16; ++chunk) {
     reduce_partials(a, rt, c_first, c_last, chunk, et, T, G, v);
     if (chunk == 0) trace_after(ts, 6, v[15]);
-    apply_epilogue<EPI>(a, ctx, red, stage, rms, rt, chunk, et, v, ts, false);
+    apply_epilogue<EPI>(a, ctx, red, stage, rms, rt, chunk, et, v, ts);
   }
   trace_at(ts, 7);
   if (et == 0) a.counters[rt] = 0;

@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const int n_pre = min(S, t_end - t_begin);
       int pt = t_begin / KT, kt = t_begin - pt * KT;
       const int kt_first = kt;
+      if (a.w_after_wait) pdl_wait();
       // weights do not depend on the previous launch: requested before its end
       for (int p = 0; p < n_pre; ++p) {
         expect(p);

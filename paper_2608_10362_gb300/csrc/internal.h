@@ -147,7 +147,7 @@ struct GemmArgs {
   int x4d;                  // are 4-D maps of the activations {64 columns, rows, planes, k tiles}
                             // with boxes of one and of gemm_small_x_group k tiles; 0: 2-D maps
                             // of the planes
-  int w_after_wait;         // gemm_small.cu, 1: the weights too are read only after
+  int w_after_wait;         // gemm_small.cu, gemm_pair.cu, 1: the weights too are read only after
                             // griddepcontrol.wait (an op-level call's weights may be anything
                             // that earlier work on the stream writes)
   int pairs;                // > 0: gemm_pair.cu's kernel with this many CTA pairs (n_pad a
@@ -181,7 +181,6 @@ struct GemmArgs {
   uint32_t* status;
   unsigned long long* trace;  // nullptr, or this op's trace row (16 slots per CTA)
   int trace_ctas;           // split epilogue kernel: CTAs (linear index) that record
-  int warm;                 // 1: dry run of the tail before griddepcontrol.wait
   int ctx_early;            // 1: every kernel before the previous one has completed when
                             // this one starts and the row-plan writer is among them, so
                             // the row plan may be read before griddepcontrol.wait
