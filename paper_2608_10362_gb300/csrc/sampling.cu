@@ -108,9 +108,10 @@ __device__ __forceinline__ Slice slice_of(const SampleArgs& a, int g, int rank, 
 }
 __device__ __forceinline__ bool in_slice(const Slice& s, int x) { return x >= 0 && x < s.end; }
 
-// NV float4 per thread and round; thread (warp w, lane l) has ids 4 l .. 4 l + 3 of
+// NV float4 per thread and round, kAhead: the next round's loads are issued before a
+// round is summed; thread (warp w, lane l) has ids 4 l .. 4 l + 3 of
 // the slice's tiles t * 16 + w, t = 0, 1, ...
-template <int NV>
+template <int NV, bool kAhead>
 __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const __grid_constant__ SampleArgs a,
                                                                           int C) {
   __shared__ ClSampleSmem sm;
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
   float best = -INFINITY;
   int arg = 0x7fffffff;
   int round = 0;
-  for (int x00 = off0; x00 - off0 < s.end - s.base; x00 += NV * kSThreads * 4, ++round) {
-    float v[NV][4];
+  constexpr int kRound = NV * kSThreads * 4;
+  auto load = [&](float (&v)[NV][4], int x00) {
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       const int x = x00 + j * kSThreads * 4;
@@ -148,6 +149,20 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[j][q] = in_slice(s, x + q) ? __ldcg(s.z + x + q) : -INFINITY;
       }
+    }
+  };
+  float nx[kAhead ? NV : 1][4];   // the next round's, under way while this one is summed
+  if constexpr (kAhead) load(nx, off0);
+  for (int x00 = off0; x00 - off0 < s.end - s.base; x00 += kRound, ++round) {
+    float v[NV][4];
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[j][q] = nx[j][q];
+      if (x00 + kRound - off0 < s.end - s.base) load(nx, x00 + kRound);
+    } else {
+      load(v, x00);
     }
     float bm = -INFINITY;
     int ba = 0x7fffffff;
@@ -318,12 +333,16 @@ __global__ void __launch_bounds__(kSThreads) accept_kernel(const __grid_constant
   accept_row<kSThreads>(a, blockIdx.x, blockIdx.y, sm, threadIdx.x, [] { __syncthreads(); });
 }
 
-// CTAs per row and float4 per thread and round (2 or 8).  A row is cut in two while
-// the launch's CTAs still fit the chip at two per SM and a CTA keeps 2048 ids.
+// CTAs per row and float4 per thread and round.  A row is cut in two while the
+// launch's CTAs still fit the chip at two per SM and a CTA keeps 2048 ids.  A slice
+// of one round is taken at once (2, or 8 for a few rows), a longer one in rounds of 4
+// with the next one's loads under way.
 // Measured (GB300, kernel alone, T = 1; before: one CTA per row, which read its row
-// twice): 1 x 32000 18.5 -> 3.3 us, 1 x 128256 57.5 -> 5.0, 32 x 128256 75.8 -> 8.3,
-// 144 x 128256 77.3 -> 20.9 (3.5 TB/s), 256 x 128256 101 -> 37.  Clusters of eight
-// whatever the row count: 144 x 128256 36 us (four waves of short CTAs); a
+// twice): 1 x 32000 18.5 -> 3.3 us, 1 x 128256 57.5 -> 4.9, 32 x 128256 75.8 -> 7.7,
+// 144 x 128256 77.3 -> 19.4 (3.8 TB/s; T = 0 13.3), 256 x 128256 101 -> 36.0; without
+// the loads ahead, rounds of 8: 7.9, 20.8, 36.7 (256 x 131071 45.8, with them 41.2), but
+// 1 x 128256 5.1 in rounds of 4.  Clusters of
+// eight whatever the row count: 144 x 128256 36 us (four waves of short CTAs); a
 // persistent grid that copies its next row while it reduces one: 35 us.
 struct SampleShape {
   int C, nv;
@@ -331,7 +350,8 @@ struct SampleShape {
 SampleShape sample_shape(int rows, int vocab) {
   int C = 1;
   while (C < kMaxCluster && rows * C * 2 <= 304 && vocab >= 2 * C * 2048) C *= 2;
-  return {C, vocab + 3 <= C * 2 * kSThreads * 4 ? 2 : 8};
+  const int round = C * kSThreads * 4;   // one float4 per thread
+  return {C, vocab + 3 <= 2 * round ? 2 : (rows <= 8 && vocab + 3 <= 8 * round ? 8 : 4)};
 }
 
 }  // namespace
@@ -352,8 +372,9 @@ cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s, bool pdl) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2 : 1;
-  return sh.nv == 2 ? cudaLaunchKernelEx(&cfg, sample_kernel<2>, a, sh.C)
-                    : cudaLaunchKernelEx(&cfg, sample_kernel<8>, a, sh.C);
+  return sh.nv == 2   ? cudaLaunchKernelEx(&cfg, sample_kernel<2, false>, a, sh.C)
+         : sh.nv == 8 ? cudaLaunchKernelEx(&cfg, sample_kernel<8, false>, a, sh.C)
+                      : cudaLaunchKernelEx(&cfg, sample_kernel<4, true>, a, sh.C);
 }
 
 cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t s, bool pdl) {
