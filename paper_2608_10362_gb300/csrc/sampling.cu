@@ -6,8 +6,8 @@
 // reading its contiguous slice of the row once.  Each of a CTA's sixteen warps
 // streams its own 128-id tiles without waiting for the others: the tiles' weight
 // sums are taken relative to that warp's maximum of the round they were loaded in.
-// Then warp 0 brings the tile sums to the slice's maximum, trades (max, first
-// argmax, weight sum) with the other slices through distributed shared memory and,
+// Then the tile sums are brought to the slice's maximum (by warp 0, or of a slice of
+// several rounds by all), and warp 0 scans them, trades (max, first argmax, sum) with the other slices through distributed shared memory and,
 // where its slice holds u * total, finds the tile and the id.  Bound by latency for
 // a few rows and by HBM for many; sample_shape() has the measurements.
 #include "internal.h"
@@ -223,6 +223,21 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
     sm.warg[w] = arg;
   }
   __syncthreads();
+  // the tile sums relative to the slice's maximum: by all threads where there are many
+  const int n_tiles = round * NV * kSWarps;
+  auto rescale = [&](int idx, float m) {   // tile (round, j, warp)
+    const float x = sm.tiles[idx];
+    return x == 0.f ? 0.f : x * __expf(sm.wmax[idx / (NV * kSWarps)][idx & (kSWarps - 1)] * it - m * it);
+  };
+  if constexpr (kAhead) {
+    if (!greedy) {
+      float m = sm.wbest[lane & (kSWarps - 1)];
+#pragma unroll
+      for (int o = kSWarps / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      for (int idx = tid; idx < n_tiles; idx += kSThreads) sm.tiles[idx] = rescale(idx, m);
+      __syncthreads();
+    }
+  }
   if (w != 0) return;
   // -------------------------------------------------- warp 0: the decision
   float u = 0.f;
@@ -237,18 +252,14 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
   float bm = sm.wbest[lane & (kSWarps - 1)];
   int ba = sm.warg[lane & (kSWarps - 1)];
   lane_argmax<kSWarps>(bm, ba);
-  // tile sums relative to the slice's maximum (a lane's tiles are consecutive), and
-  // their scan
-  const int tpl = (round * NV * kSWarps + 31) / 32;
-  float* tw = sm.tiles + lane * tpl;
+  // the scan of the tile sums (a lane's tiles are consecutive)
+  const int tpl = (n_tiles + 31) / 32;
   float ls = 0.f, excl = 0.f, incl = 0.f;
   if (!greedy) {
     for (int t = 0; t < tpl; ++t) {
-      const int idx = lane * tpl + t;   // tile (round, j, warp)
-      const float x = tw[t];
-      const float y = x == 0.f ? 0.f : x * __expf(sm.wmax[idx / (NV * kSWarps)][idx & (kSWarps - 1)] * it - bm * it);
-      tw[t] = y;
-      ls += y;
+      const int idx = lane * tpl + t;
+      if constexpr (!kAhead) sm.tiles[idx] = rescale(idx, bm);
+      ls += sm.tiles[idx];
     }
     lane_scan(ls, lane, excl, incl);
   }
@@ -293,7 +304,7 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
       if (lane == src) {   // the first tile whose running sum passes r, else the last with mass
         float cum = excl;
         for (int k = 0; k < tpl; ++k) {
-          const float y = tw[k];
+          const float y = sm.tiles[src * tpl + k];
           if (y > 0.f) {
             sel = src * tpl + k;
             before = cum;
@@ -339,9 +350,10 @@ __global__ void __launch_bounds__(kSThreads) accept_kernel(const __grid_constant
 // with the next one's loads under way.
 // Measured (GB300, kernel alone, T = 1; before: one CTA per row, which read its row
 // twice): 1 x 32000 18.5 -> 3.3 us, 1 x 128256 57.5 -> 4.9, 32 x 128256 75.8 -> 7.7,
-// 144 x 128256 77.3 -> 19.4 (3.8 TB/s; T = 0 13.3), 256 x 128256 101 -> 36.0; without
-// the loads ahead, rounds of 8: 7.9, 20.8, 36.7 (256 x 131071 45.8, with them 41.2), but
-// 1 x 128256 5.1 in rounds of 4.  Clusters of
+// 144 x 128256 77.3 -> 18.6 (4.0 TB/s; T = 0 13.2), 256 x 128256 101 -> 33.6.  With the
+// tile sums rescaled by warp 0 alone 19.4 and 36.0; without the loads ahead too, rounds
+// of 8, 20.8 and 36.7 - but 1 x 128256 5.1 in rounds of 4.  The scan over the tiles by all
+// warps took 17.9 and 30.8, but adds them in another order.  Clusters of
 // eight whatever the row count: 144 x 128256 36 us (four waves of short CTAs); a
 // persistent grid that copies its next row while it reduces one: 35 us.
 struct SampleShape {
