@@ -7,9 +7,10 @@
 // streams its own 128-id tiles without waiting for the others: the tiles' weight
 // sums are taken relative to that warp's maximum of the round they were loaded in.
 // Then the tile sums are brought to the slice's maximum (by warp 0, or of a slice of
-// several rounds by all), and warp 0 scans them, trades (max, first argmax, sum) with the other slices through distributed shared memory and,
-// where its slice holds u * total, finds the tile and the id.  Bound by latency for
-// a few rows and by HBM for many; sample_shape() has the measurements.
+// several rounds by all), and warp 0 scans them, trades (max, first argmax, sum) with
+// the other slices through distributed shared memory and, where its slice holds
+// u * total, finds the tile and the id.  Bound by latency for a few rows and by HBM for
+// many; sample_shape() has the measurements.
 #include "internal.h"
 #include "ptx.cuh"
 #include "sample_body.cuh"
@@ -109,8 +110,8 @@ __device__ __forceinline__ Slice slice_of(const SampleArgs& a, int g, int rank, 
 __device__ __forceinline__ bool in_slice(const Slice& s, int x) { return x >= 0 && x < s.end; }
 
 // NV float4 per thread and round, kAhead: the next round's loads are issued before a
-// round is summed; thread (warp w, lane l) has ids 4 l .. 4 l + 3 of
-// the slice's tiles t * 16 + w, t = 0, 1, ...
+// round is summed; thread (warp w, lane l) has ids 4 l .. 4 l + 3 of the slice's tiles
+// t * 16 + w, t = 0, 1, ...
 template <int NV, bool kAhead>
 __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const __grid_constant__ SampleArgs a,
                                                                           int C) {
