@@ -896,8 +896,8 @@ def run_case(args):
 
 TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "verify_7b_2layers_k4_ctx2048_dram.md")
 # the sources of the kernels a verify pass launches (and of their launch set-up)
-VERIFY_SOURCES = ("api.cu", "attention.cu", "attn_body.cuh", "embed.cu", "embed_body.cuh", "gemm.cu",
-                  "gemm_epi.cuh", "internal.h", "pack.cu", "ptx.cuh")
+VERIFY_SOURCES = ("api.cu", "attn_tc.cu", "embed.cu", "embed_body.cuh", "gemm_epi.cuh", "gemm_small.cu",
+                  "internal.h", "pack.cu", "ptx.cuh")
 
 
 def kernel_sources_hash(names=VERIFY_SOURCES) -> str:

@@ -46,11 +46,10 @@
 // through its own ring of D = 2 record slots with cp.async, one commit group
 // per record (small copies: per-request cost decides, and 1 KB bulk copies
 // were slower).  Rings of 3, 4 and 6 slots are no faster (GB300, 12288 x 4096 at 5 rows:
-// 8.9 us with 2, 9.2 with 3 or 4): a record costs an SM 62 cycles, most of them its
-// unpacking and MMAs (with the loads from one place alone 8.7 us, without the
-// arithmetic 7.0; ALU pipe 48%, issue 46% busy), where HBM would allow 46.  Tried
-// instead: a warp per column range with its activations in registers and the records
-// loaded straight to registers, 9.8 us; two CTAs per SM 9.5.  The
+// 8.9 us with 2, 9.2 with 3 or 4): a record costs an SM 62 cycles where HBM would allow
+// 46.  Tried instead: two CTAs per SM, 9.5 us; a warp per column range with its
+// activations in registers and the records loaded straight to registers, 9.8 (8.7 of it
+// with every record in L2: unpacking and MMAs, ALU pipe 48% and issue 46% busy).  The
 // activations arrive as one 1-D bulk copy (TMA) per row, outside the load/store unit's
 // queue.  That wait is bounded: on expiry the kernel sets bit 0 of the optional status
 // word and finishes without computing.  A tile a warp covers whole is stored directly;
