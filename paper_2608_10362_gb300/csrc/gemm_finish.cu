@@ -1,5 +1,5 @@
-// gemm_finish.cu - the second launch of a GEMM over more than 16 activation rows:
-// sums the stream-K partials of a row tile and runs the fused epilogue.
+// gemm_finish.cu - the second launch of a GEMM over more activation rows than
+// gemm_small.cu takes: sums the stream-K partials of a row tile and runs the epilogue.
 //
 // CTA (row tile, 16-row chunk), 128 threads; the sums are formed with a thread per
 // feature of the tile, then the tile is turned in shared memory and a thread finishes
