@@ -10,7 +10,9 @@
 // several rounds by all), and warp 0 scans them, trades (max, first argmax, sum) with
 // the other slices through distributed shared memory and, where its slice holds
 // u * total, finds the tile and the id.  Bound by latency for a few rows and by HBM for
-// many; sample_shape() has the measurements.
+// many; sample_shape() has the measurements.  Ids that differ from the ones of 64-bit
+// sums (u within a rounding of a boundary): 25 of 11232 over five shapes of 64 to 256
+// rows, with one CTA per row 25.
 #include "internal.h"
 #include "ptx.cuh"
 #include "sample_body.cuh"
