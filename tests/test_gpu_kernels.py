@@ -157,10 +157,12 @@ def test_sampler_slices(rows, vocab, offset):
                 assert T > 0 and abs(u[r] - c[min(out[r], expect)]) < 1e-5, (r, T, out[r], expect)
 
 
-def test_sampler_degenerate_rows():
+@pytest.mark.parametrize("copies", [1, 40])
+def test_sampler_degenerate_rows(copies):
     """Rows without a proper distribution: a NaN among the logits, +inf, every
     logit -inf but one, all equal; the draw is an id of the row (the first argmax
-    where the weights have no finite sum)."""
+    where the weights have no finite sum).  Few rows (slices of one round) and many
+    (slices of several)."""
     from paper_2608_10362_gb300 import op_sample
     V = 32000
     z = gen_logits(22, 5, V, scale=1.0)
@@ -169,11 +171,16 @@ def test_sampler_degenerate_rows():
     z[2, :] = -np.inf
     z[2, 31999] = -3.0
     z[3, :] = 0.0
-    u = np.full(5, 0.5, dtype=np.float32)
-    out = op_sample(torch.from_numpy(z).cuda(), 1.0, torch.from_numpy(u).cuda()).cpu().numpy()
+    u = np.full(5 * copies, 0.5, dtype=np.float32)
+    zt = torch.from_numpy(np.tile(z, (copies, 1))).cuda()
+    out = op_sample(zt, 1.0, torch.from_numpy(u).cuda()).cpu().numpy().reshape(copies, 5)
+    assert (out == out[0]).all()
+    out = out[0]
     assert out[0] == int(np.nanargmax(z[0])) and out[1] == 29000 and out[2] == 31999
     assert abs(int(out[3]) - V // 2) <= 1
-    g = op_sample(torch.from_numpy(z).cuda(), 0.0).cpu().numpy()
+    g = op_sample(zt, 0.0).cpu().numpy().reshape(copies, 5)
+    assert (g == g[0]).all()
+    g = g[0]
     assert g[0] == int(np.nanargmax(z[0])) and g[1] == 29000 and g[2] == 31999 and g[3] == 0
 
 
