@@ -15,8 +15,8 @@
 extern "C" {
 #endif
 
-/* Scratch bytes that memspec_op_linear needs for (rows, n_out, k): split-K
- * partial sums and per-row-tile arrival counters. */
+/* Scratch bytes that memspec_op_linear needs for (rows, n_out, k): arrival
+ * counters and split-K partial sums. */
 memspec_status memspec_op_linear_scratch_bytes(int32_t rows, int32_t n_out, int32_t k,
                                                size_t* bytes);
 
@@ -28,8 +28,10 @@ memspec_status memspec_op_linear_scratch_bytes(int32_t rows, int32_t n_out, int3
  * on the same stream, one CTA per row tile and 16-row chunk).
  * rows in 1..256, k a multiple of 8, n_out >= 1, and
  * ceil(n_out/128) * ceil(k/64) * (SMs + 1) below 2^32.
- * scratch_dev: memspec_op_linear_scratch_bytes bytes, 256-byte aligned; its
- * counters must be zero on entry and are left zero on exit (zero it once).
+ * scratch_dev: memspec_op_linear_scratch_bytes bytes, 256-byte aligned, zeroed
+ * once before its first use.  One scratch of the largest call's size serves
+ * calls of any sizes that run one after another; calls that may overlap (other
+ * streams) need scratches of their own.
  * status_dev: uint32 device word, bits set on in-kernel errors (may be NULL).
  * x, w: 16-byte aligned.  Errors: INVALID_ARG, UNSUPPORTED, CUDA. */
 memspec_status memspec_op_linear(const void* x_dev, const void* w_dev, float* y_dev,

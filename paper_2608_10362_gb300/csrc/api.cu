@@ -550,7 +550,7 @@ size_t layout_workspace(const memspec_init_params* p, memspec_ctx* c, uint8_t* b
   const int proj_rt = std::max({ceil_div(fmax, 64), ceil_div(model_q(t) + 2 * model_kv(t), 128),
                                 has_draft ? ceil_div(model_q(dm) + 2 * model_kv(dm), 128) : 1, ceil_div(dmax, 128)});
   const size_t o_gp = w.take(static_cast<size_t>(std::max(2 * nsm, proj_rt + 1 + nsm)) * kMaxRows * 128 * 4);
-  const size_t o_gc = w.take(static_cast<size_t>(max_rt) * 4);   // split-K arrival counters
+  const size_t o_gc = w.take(static_cast<size_t>(std::max(max_rt, nsm)) * 4);   // split-K arrival counters
   const size_t o_apo = w.take(po * 4);
   const size_t o_apml = w.take(po / 64 * 2 * 4 + 1024);
   const size_t o_acnt = w.take(cnt * 4);
@@ -2243,18 +2243,18 @@ void memspec::set_op_error(const char* msg) { g_op_error = msg; }
 
 extern "C" {
 
-static size_t op_linear_scratch(int rows, int n_out, int k) {
-  const int n_pad = round_up(rows, 16);
-  const int rt = ceil_div(n_out, 128);
-  (void)k;
-  // partials, then one arrival counter per row tile
-  return align256(static_cast<size_t>(2) * sm_count() * n_pad * 128 * 4) +
-         align256(static_cast<size_t>(rt) * 4) + 256;
+// memspec_op_linear's scratch: an arrival counter per CTA and a status word in a head
+// of one size for all calls, then the partials.  Callers zero a scratch once and use it
+// for calls of any sizes: no call's partials may reach another's counters.
+static size_t op_linear_counter_bytes() { return align256(static_cast<size_t>(sm_count()) * 4); }
+static size_t op_linear_head() { return op_linear_counter_bytes() + 256; }
+static size_t op_linear_scratch(int rows) {
+  return op_linear_head() + static_cast<size_t>(2) * sm_count() * round_up(rows, 16) * 128 * 4;
 }
 
 memspec_status memspec_op_linear_scratch_bytes(int32_t rows, int32_t n_out, int32_t k, size_t* bytes) {
   if (bytes == nullptr || rows < 1 || rows > kMaxRows || n_out < 1 || k < 8) return MEMSPEC_ERR_INVALID_ARG;
-  *bytes = op_linear_scratch(rows, n_out, k);
+  *bytes = op_linear_scratch(rows);
   return MEMSPEC_OK;
 }
 
@@ -2304,7 +2304,7 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
     g_op_error = "x and w must be 16-byte aligned, scratch 256-byte aligned";
     return MEMSPEC_ERR_INVALID_ARG;
   }
-  if (scratch_bytes < op_linear_scratch(rows, n_out, k)) {
+  if (scratch_bytes < op_linear_scratch(rows)) {
     g_op_error = "scratch too small";
     return MEMSPEC_ERR_INVALID_ARG;
   }
@@ -2328,12 +2328,9 @@ memspec_status memspec_op_linear(const void* x, const void* w, float* y, int32_t
   a.out = y;
   a.out_ld = n_out;
   uint8_t* sb = static_cast<uint8_t*>(scratch);
-  a.partials = reinterpret_cast<float*>(sb);
-  const size_t part_bytes = align256(static_cast<size_t>(2) * sm_count() * n_pad * 128 * 4);
-  a.counters = reinterpret_cast<int*>(sb + part_bytes);
-  a.status = status != nullptr ? status
-                               : reinterpret_cast<uint32_t*>(sb + part_bytes +
-                                                             align256(static_cast<size_t>(a.row_tiles) * 4));
+  a.counters = reinterpret_cast<int*>(sb);
+  a.status = status != nullptr ? status : reinterpret_cast<uint32_t*>(sb + op_linear_counter_bytes());
+  a.partials = reinterpret_cast<float*>(sb + op_linear_head());
   a.plan = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // set-up overlaps the previous kernel's end; every read, the weights' too, comes after it

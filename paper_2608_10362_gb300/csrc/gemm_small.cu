@@ -618,8 +618,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_small_kernel(const __grid_co
           // loads (which bypass L1).
           named_bar_sync(1, 128);
           if (et == 0) {
-            ctl.reduce_flag = atom_add_acq_rel_gpu(&a.counters[rt], 1) == c_last - c_first ? 1 : 0;
-            if (ctl.reduce_flag) a.counters[rt] = 0;
+            // counted at the first contributor, whose range ends in this tile: no other
+            // split tile has the same one
+            ctl.reduce_flag = atom_add_acq_rel_gpu(&a.counters[c_first], 1) == c_last - c_first ? 1 : 0;
+            if (ctl.reduce_flag) a.counters[c_first] = 0;
           }
           named_bar_sync(1, 128);
           trace_at(ts, 5);

@@ -139,7 +139,8 @@ struct GemmArgs {
   float eps;
   // split-K scratch
   float* partials;          // gemm.cu: [2 * grid][n_pad * 128]; gemm_pair.cu: pair_slot
-  int* counters;            // [row_tiles], zero on entry, left zero
+  int* counters;            // zero on entry, left zero: gemm.cu and pass.cu [row_tiles],
+                            // gemm_small.cu [grid]
   int split_epi;            // 1: contributors to a split row tile only store their partials;
                             // gemm_split_epi_kernel (the next launch) sums them and runs the
                             // epilogue, one CTA per (row tile, 16-row chunk)

@@ -375,7 +375,9 @@ def op_linear(x: torch.Tensor, w: torch.Tensor, scratch: torch.Tensor | None = N
     nb = _linear_scratch_bytes(rows, n_out, k)
     if scratch is None:
         scratch = torch.zeros(nb + 256, dtype=torch.uint8, device=x.device)
-    base = (scratch.data_ptr() + 255) & ~255
+    start = scratch.data_ptr()
+    base = (start + 255) & ~255
+    nb = max(0, scratch.nbytes - (base - start))
     y = torch.empty((rows, n_out), dtype=torch.float32, device=x.device)
     st = lib.memspec_op_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, n_out, k, base, nb, None,
                                _raw_stream(x, stream))

@@ -1,6 +1,8 @@
 """Kernel-level parity on the GPU (through the C ABI): the weight-streaming GEMM,
 the categorical sampler, and the acceptance / resample / commit kernel fed with
 synthetic logits, against the oracle's definitions."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -42,6 +44,52 @@ def test_linear_matches_fp64_matmul(rows, n_out, k):
     # a second launch reuses the same scratch: counters must have been reset
     y2 = op_linear(xt, wt).cpu().numpy().astype(np.float64)
     np.testing.assert_array_equal(y, y2)      # deterministic split-K reduction
+
+
+def test_linear_calls_of_all_row_counts_share_one_scratch():
+    """One scratch, zeroed once, for calls of every row count and size in turn, as a
+    program keeps it for its projections.  The calls of up to 16 rows are of sizes
+    whose split row tiles no cluster holds (12, 48 and 24 row tiles of 47 k tiles), so
+    that they count arrivals in the scratch; the others leave partial sums in it.  y is
+    full of NaN before each call: a row tile that no CTA finishes shows."""
+    from paper_2608_10362_gb300 import _lib
+    lib = _lib.load()
+    sizes = [(5, 1500, 3000), (32, 12288, 4096), (5, 1500, 3000), (200, 12288, 4096), (16, 6100, 3000),
+             (256, 300, 4096), (1, 3000, 3000), (17, 40000, 1000), (5, 1500, 3000), (16, 40000, 72), (5, 6100, 3000)]
+    need = C.c_size_t()
+    nbytes = 0
+    for rows, n_out, k in sizes:
+        assert lib.memspec_op_linear_scratch_bytes(rows, n_out, k, C.byref(need)) == 0
+        nbytes = max(nbytes, need.value)
+    scratch = torch.zeros(nbytes + 256, dtype=torch.uint8, device="cuda")
+    base = (scratch.data_ptr() + 255) // 256 * 256
+    g = torch.Generator(device="cuda").manual_seed(8)
+    for rows, n_out, k in sizes:
+        x = torch.randn(rows, k, device="cuda", generator=g).to(torch.bfloat16)
+        w = (torch.randn(n_out, k, device="cuda", generator=g) * 0.02).to(torch.bfloat16)
+        y = torch.full((rows, n_out), float("nan"), device="cuda")
+        st = lib.memspec_op_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, n_out, k, base, nbytes, None,
+                                   torch.cuda.current_stream().cuda_stream)
+        assert st == 0, lib.memspec_op_last_error()
+        x, w = x.double(), w.double()
+        bad = ~((y.double() - x @ w.T).abs() <= 1e-4 * (x.abs() @ w.abs().T) + 1e-6)   # true for NaN
+        assert not bad.any(), (rows, n_out, k, int(bad.sum()))
+
+
+def test_linear_refuses_a_scratch_that_is_too_small():
+    """The call is given what the scratch holds from its first 256-byte boundary on."""
+    from paper_2608_10362_gb300 import MemSpecError, _lib, op_linear
+    need = C.c_size_t()
+    assert _lib.load().memspec_op_linear_scratch_bytes(32, 256, 64, C.byref(need)) == 0
+    x = torch.ones(32, 64, dtype=torch.bfloat16, device="cuda")
+    w = torch.ones(256, 64, dtype=torch.bfloat16, device="cuda")
+    buf = torch.zeros(need.value + 512, dtype=torch.uint8, device="cuda")
+    assert buf.data_ptr() % 256 == 0
+    assert (op_linear(x, w, buf[:need.value]) == 64).all()
+    assert (op_linear(x, w, buf[1:256 + need.value]) == 64).all()
+    for small in (buf[:need.value - 1], buf[1:need.value + 255], buf[1:9]):
+        with pytest.raises(MemSpecError):
+            op_linear(x, w, small)
 
 
 @pytest.mark.parametrize("n_out,k", [(12288, 4096), (4096, 11008), (32000, 4096)])
