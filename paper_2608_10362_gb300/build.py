@@ -19,7 +19,8 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libmemspec.so")
 SOURCES = ["gemm.cu", "gemm_pair.cu", "gemm_finish.cu", "gemm_small.cu", "attention.cu", "attn_tc.cu", "embed.cu", "sampling.cu", "api.cu", "noalloc.cu", "pass.cu", "pack.cu", "tree.cu",
            "draft_fused.cu", "sched.cpp", "int4.cu"]
-HEADERS = ["ptx.cuh", "internal.h", "gemm_epi.cuh", "attn_body.cuh", "sample_body.cuh", "embed_body.cuh", "pass.h"]
+HEADERS = ["ptx.cuh", "internal.h", "gemm_epi.cuh", "attn_body.cuh", "sample_body.cuh", "embed_body.cuh", "pass.h",
+           "first_use.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

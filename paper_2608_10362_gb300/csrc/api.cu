@@ -21,6 +21,7 @@
 
 #include "../../include/memspec.h"
 #include "../../include/memspec_ops.h"
+#include "first_use.h"
 #include "internal.h"
 #include "pass.h"
 
@@ -1259,6 +1260,28 @@ memspec_status launch_table(memspec_ctx* c, const OpTable& t) {
   return MEMSPEC_OK;
 }
 
+// Why a step's first use cannot be captured on this stream: it is part of a capture of
+// the caller's, whose graph would take the step's plain launches, or it is the legacy
+// default stream.  Found out before anything runs.
+cudaError_t not_capturable(cudaStream_t s) {
+  if (s == nullptr || s == cudaStreamLegacy) return cudaErrorStreamCaptureUnsupported;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &st);
+  return e == cudaSuccess && st != cudaStreamCaptureStatusNone ? cudaErrorIllegalState : e;
+}
+
+// run_then_capture's CUDA calls.
+struct StreamGraphs {
+  using Graph = cudaGraph_t;
+  using Exec = cudaGraphExec_t;
+  cudaStream_t stream;
+  bool begin() { return cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess; }
+  bool end(Graph* g) { return cudaStreamEndCapture(stream, g) == cudaSuccess; }
+  bool instantiate(Exec* x, Graph g) { return cudaGraphInstantiate(x, g, 0) == cudaSuccess; }
+  void destroy(Graph g) { cudaGraphDestroy(g); }
+  void clear_error() { (void)cudaGetLastError(); }
+};
+
 // Build the op list, then run it: one persistent launch (pass kernel) or one
 // launch per op; captured once as a CUDA graph per key and replayed when graphs
 // are on.  `use_pass` = false always runs separate launches.
@@ -1274,6 +1297,7 @@ memspec_status run_pass(memspec_ctx* c, const GraphKey& key, bool use_pass, Emit
       c->last_launches[slot] = c->graph_launches[key];
       return MEMSPEC_OK;
     }
+    if (cudaError_t e = not_capturable(c->main); e != cudaSuccess) return cuda_fail(c, e, "begin capture");
   }
   std::vector<PassOp> ops;
   memspec_status s = emit(ops);
@@ -1292,16 +1316,19 @@ memspec_status run_pass(memspec_ctx* c, const GraphKey& key, bool use_pass, Emit
     if (s != MEMSPEC_OK) return s;
   }
   if (!c->p.use_graphs) return pass ? launch_table(c, t) : run_ops_separately(c, ops);
-  // The first use runs as plain launches and is captured for the next ones while the
-  // GPU is at work: capturing 250 launches before the first of them runs would hold a
-  // request's first step for a millisecond.
   if (!pass) {
-    s = run_ops_separately(c, ops);
-    if (s != MEMSPEC_OK) return s;
+    StreamGraphs cu{c->main};
+    cudaGraphExec_t ex = nullptr;
+    s = run_then_capture(cu, [&] { return run_ops_separately(c, ops); }, &ex);
+    if (ex != nullptr) {
+      c->graphs.emplace(key, ex);
+      c->graph_launches[key] = n_launch;
+    }
+    return s;
   }
   cudaError_t e = cudaStreamBeginCapture(c->main, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(c, e, "begin capture");
-  s = pass ? launch_table(c, t) : run_ops_separately(c, ops);
+  s = launch_table(c, t);
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->main, &g);
   if (s != MEMSPEC_OK) {
@@ -1315,7 +1342,6 @@ memspec_status run_pass(memspec_ctx* c, const GraphKey& key, bool use_pass, Emit
   if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
   c->graphs.emplace(key, ex);
   c->graph_launches[key] = n_launch;
-  if (!pass) return MEMSPEC_OK;
   e = cudaGraphLaunch(ex, c->main);
   if (e != cudaSuccess) return cuda_fail(c, e, "graph launch");
   return MEMSPEC_OK;

@@ -8,6 +8,7 @@ every access stays in bounds.  A host-side wait that runs out returns
 MEMSPEC_ERR_TIMEOUT while the stream keeps running a finite kernel.
 """
 import ctypes as C
+import warnings
 
 import numpy as np
 import pytest
@@ -51,6 +52,35 @@ def _clean_step_after(eng, to, do, seed):
     eng.step(4, 1.0, eng.results_host)
     check_step(eng, sd, 4, 1.0, seed, 0, rep)
     assert rep.band_flags == 0
+
+
+def test_first_use_inside_a_callers_capture_is_refused(tiny_engine):
+    """A step shape's first use while the caller captures the main stream: an error,
+    and none of the step's launches in the caller's graph (its replay leaves the
+    logits as they are); the next use outside runs as ever."""
+    from paper_2608_10362_gb300 import MemSpecError, _lib
+    eng, _, _ = tiny_engine
+    eng.prefill(0, gen_prompt(7, 40, 2048), seed=1)
+    eng.write_buffer(_lib.BUF_DRAFT_TOKENS, gen_prompt(8, 3, 2048).astype(np.int32)[None])
+    eng.set_batch(1)
+    mark = np.full((1, 4, 2048), 12.5, np.float32)
+    eng.write_buffer(_lib.BUF_TARGET_LOGITS, mark)
+    graph = torch.cuda.CUDAGraph()
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")        # the graph is empty
+        with torch.cuda.graph(graph, stream=eng.stream, capture_error_mode="thread_local"):
+            with pytest.raises(MemSpecError):
+                eng.verify_step(3)             # K = 3: no other test of this engine has used it
+    graph.replay()
+    torch.cuda.synchronize()
+    assert eng.sync() == 0
+    assert np.array_equal(eng.target_logits(1, 3), mark)
+    logits = []
+    for _ in range(2):                         # plain launches, then the captured ones
+        eng.verify_step(3)
+        assert eng.sync() == 0
+        logits.append(eng.target_logits(1, 3).copy())
+    assert np.array_equal(logits[0], logits[1]) and np.abs(logits[0]).max() < 12.5
 
 
 def test_out_of_range_token_is_reported(tiny_engine):
