@@ -969,6 +969,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       if (!pass_x(c, a, pass, c->xg, c->xg_lo, rows, d, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
+      a.apart = prefill;
       a.rms = 1;
       a.ss = c->ss;
       a.ss_count = ss_count;
@@ -1046,6 +1047,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       if (!pass_x(c, a, pass, c->o, c->o_lo, rows, qd, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
+      a.apart = prefill;
       a.epi = EPI_RESIDUAL;
       a.h = c->h;
       a.h_ld = d;
@@ -1072,6 +1074,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       if (!pass_x(c, a, pass, c->xg, c->xg_lo, rows, d, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
+      a.apart = prefill;
       a.rms = 1;
       a.ss = c->ss;
       a.ss_count = ss_count;
@@ -1097,6 +1100,7 @@ memspec_status emit_forward(memspec_ctx* c, ModelRT& m, const FwdSpec& f,
       if (!pass_x(c, a, pass, c->act, c->act_lo, rows, F, n_pad))
         return fail(c, MEMSPEC_ERR_CUDA, "activation tensor map");
       a.split = 1;
+      a.apart = prefill;
       a.epi = EPI_RESIDUAL;
       a.h = c->h;
       a.h_ld = d;
@@ -1386,7 +1390,7 @@ memspec_status draft_wait_ready(memspec_ctx* c, DraftRec& dr) {
 
 // Keys and values of positions [from, to) of request `req`, in passes of up to
 // kPrefillChunk rows, the last of as many as are left.  (2047 positions of the 7B, ms:
-// passes of 256 rows 48.5, 192 55.4, 128 65.4.)
+// passes of 256 rows 47.9, 192 53.6, 128 62.8.)
 memspec_status prefill_range(memspec_ctx* c, ModelRT& m, int req, int from, int to) {
   for (int start = from; start < to; start += kPrefillChunk) {
     FwdSpec f{};

@@ -9,15 +9,23 @@
 // half as large and the activation traffic is halved:
 //   one plane                  N = n_pad,     CTA r loads rows [r n_pad/2, + n_pad/2)
 //   hi + lo, 2 n_pad <= 256    N = 2 n_pad,   CTA 0 loads the hi plane, CTA 1 the lo
-//   hi + lo, larger            N = n_pad twice into one accumulator, halves of both
-// Each CTA's tensor memory receives its own 128 features, in gemm.cu's accumulator
-// layout.
+//   hi + lo, larger            N = n_pad twice, halves of both: into one accumulator, or
+//                              (prefill) two that are added at the end
+// Each CTA's tensor memory receives its own 128 features.  In one accumulator the chain
+// of sums is twice as long and a lo product, 2^-9 of its hi product, is cut at the hi
+// sum's last bit: of a 256-row pass's V (d = 4096) 1.36e-3 of the values are not the
+// rounded 64-bit ones, with two 0.67e-3, as with 128 rows side by side.  Two fill the
+// tensor memory, so that a segment's MMAs wait until the last one's sums are drained: 2047
+// prompt tokens of the 7B 48.1 ms (with one 46.9), 8 layers of the 8B verify of 144 rows
+// 1.37 (1.30; with 32 columns of both planes per load in the drain no less: the stores
+// bound it).  Prefill takes two, so that its keys and values are as exact in passes of 256
+// rows as in passes of 128.
 //
 // Roles (192 threads per CTA): warp 0 copies its CTA's weights and half of the
 // activations, both CTAs' bytes completing on CTA 0's barrier (.cta_group::2; a
 // thread of CTA 1 that passed its own barrier on with a release arrive held the
 // loop at 1 us per tile); warp 1 of CTA 0 issues every MMA; warps 2-5 drain the
-// accumulator (double-buffered).  Stream-K over pairs; split tiles are left as fp32
+// accumulator (double-buffered where two fit).  Stream-K over pairs; split tiles are left as fp32
 // partials for gemm_finish.cu, and so are whole ones but those of the fp32-output
 // epilogue (a fused epilogue in here, by four warps, took 20 us for a whole tile of
 // 144 rows at the end of some CTAs' ranges).  Every wait is bounded.
@@ -29,6 +37,7 @@
 //   7B target, 128 rows  gate/up 63.2 / 33.0 (5.5 TB/s), QKV 29.0 / 20.5, down 32.5 /
 //                        23.3, O 13.3 / 10.4; finishing 9-15 / 5-6.5
 //   7B target, 256 rows  gate/up 48 (1.9 PFLOP/s), QKV 29 (1.8), down 28 (1.6), O 15.5
+//                        (one accumulator; prefill's two take 1 to 1.5 more)
 #include <cuda_bf16.h>
 
 #include "gemm_epi.cuh"
@@ -98,8 +107,10 @@ __device__ __forceinline__ void arrive_at(uint64_t* bar, uint32_t rank) {
                : "memory");
 }
 
-__host__ __device__ inline int pair_layout(int n_pad, int split) {
-  return !split ? kPlain : (2 * n_pad <= 256 ? kWide : kTwice);
+// hi and lo planes as two MMAs, accumulator columns as kWide's
+constexpr int kApart = 3;
+__host__ __device__ inline int pair_layout(int n_pad, int split, int apart) {
+  return !split ? kPlain : (2 * n_pad <= 256 ? kWide : (apart ? kApart : kTwice));
 }
 // activation bytes of one stage in one CTA
 __host__ __device__ inline int pair_b_bytes(int n_pad, int split) { return n_pad * (split ? 128 : 64); }
@@ -148,9 +159,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   const int T = (a.row_tiles + 1) / 2 * KT;      // tiles of row-tile pairs
   const int G = gridDim.x >> 1, c = blockIdx.x >> 1;
   const int t_begin = sk_begin(c, T, G), t_end = sk_begin(c + 1, T, G);
-  const int layout = pair_layout(a.n_pad, a.split);
-  const int acols = acc_cols(a, layout);
-  const uint32_t tmem_cols = tmem_cols_for(acols);
+  const int layout = pair_layout(a.n_pad, a.split, a.apart);
+  const bool sums = layout == kWide || layout == kApart;   // hi in columns [0, n_pad), lo in the next n_pad
+  const int acols = sums ? 2 * a.n_pad : a.n_pad;
+  const int bufs = layout == kApart ? 1 : 2;               // accumulators that fit (512 columns)
+  const uint32_t tmem_cols = layout == kApart ? 512 : tmem_cols_for(acols);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -274,16 +287,18 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const uint64_t adesc0 = make_smem_desc_sw128(smem_addr(smem_a));
       const uint64_t bdesc0 = make_smem_desc_sw128(smem_addr(smem_b));
       const uint32_t a_step = kABytes >> 4, b_step = static_cast<uint32_t>(b_bytes) >> 4;
-      const uint32_t p_step = static_cast<uint32_t>(a.n_pad / 2 * 128) >> 4;   // kTwice: the lo plane
+      // kTwice, kApart: the lo plane and its accumulator
+      const uint32_t p_step = static_cast<uint32_t>(a.n_pad / 2 * 128) >> 4;
+      const uint32_t lo_col = layout == kApart ? a.n_pad : 0;
       int s = 0, seg = 0;
       uint32_t ph = 0;
       bool ok = true;
       for (int t = t_begin; t < t_end && ok; ++seg) {
         const int seg_end = min(t_end, (t / KT + 1) * KT);
-        const int buf = seg & 1;
-        if (seg >= 2) {
+        const int buf = seg & (bufs - 1), use = seg >> (bufs - 1);
+        if (use > 0) {
           ok = __all_sync(0xffffffffu,
-                          mbar_wait_cluster_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>((seg >> 1) - 1) & 1u,
+                          mbar_wait_cluster_bounded(&ctl.acc_empty[buf], static_cast<uint32_t>(use - 1) & 1u,
                                                     abort_flag, a.status));
           if (!ok) break;
         }
@@ -298,7 +313,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           const uint32_t acc0 = tt > t ? 1u : 0u;
           if (lead) {
             if (tt == t_begin) trace_at(trace, 3);
-            if (layout != kTwice) {
+            if (layout < kTwice) {
 #pragma unroll
               for (int kk = 0; kk < kTileK / 16; ++kk)
                 mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
@@ -306,7 +321,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
 #pragma unroll
               for (int kk = 0; kk < kTileK / 16; ++kk) {
                 mma_pair(d_tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-                mma_pair(d_tmem, ad + 2 * kk, bd + p_step + 2 * kk, idesc, 1u);
+                mma_pair(d_tmem + lo_col, ad + 2 * kk, bd + p_step + 2 * kk, idesc, kk > 0 || lo_col == 0 ? 1u : acc0);
               }
             }
             commit_pair(&ctl.empty[s]);
@@ -343,10 +358,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const int seg_end = min(t_end, (pt + 1) * KT);
       [[maybe_unused]] const bool whole = t == pt * KT && seg_end == (pt + 1) * KT;
       const int slot = pair_slot(a, pt, c, rank, seg == 0 ? 0 : 1);
-      const int buf = seg & 1;
+      const int buf = seg & (bufs - 1);
       if (threadIdx.x == 64)
         ctl.wait_ok =
-            mbar_wait_bounded(&ctl.acc_full[buf], static_cast<uint32_t>(seg >> 1) & 1u, abort_flag, a.status) ? 1 : 0;
+            mbar_wait_bounded(&ctl.acc_full[buf], static_cast<uint32_t>(seg >> (bufs - 1)) & 1u, abort_flag, a.status) ? 1 : 0;
       named_bar_sync(1, 128);
       const int ok = ctl.wait_ok;
       named_bar_sync(1, 128);
@@ -358,7 +373,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         const int chunks = (a.rows_total + 15) / 16;
         for (int chunk = 0; chunk < chunks; ++chunk) {
           float v[16];
-          tmem_ld_sum(tbase + chunk * 16, layout == kWide ? a.n_pad : 0, v);
+          tmem_ld_sum(tbase + chunk * 16, sums ? a.n_pad : 0, v);
           if constexpr (F32) {
             if (whole) {
               const int f = rt * kTileM + et;
@@ -421,7 +436,7 @@ int gemm_pair_pad(int rows, int split) {
 }
 
 int gemm_pair_box_rows(int n_pad, int split) {
-  return pair_layout(n_pad, split) == kWide ? n_pad : n_pad / 2;
+  return pair_layout(n_pad, split, 0) == kWide ? n_pad : n_pad / 2;
 }
 
 int gemm_pair_stages(int n_pad, int split, int epi) {

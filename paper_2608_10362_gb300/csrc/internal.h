@@ -153,6 +153,8 @@ struct GemmArgs {
                             // that earlier work on the stream writes)
   int pairs;                // > 0: gemm_pair.cu's kernel with this many CTA pairs (n_pad a
                             // = gemm_pair_pad, map_b boxes of gemm_pair_box_rows rows)
+  int apart;                // gemm_pair.cu, 1: over more than 128 rows too the planes have
+                            // accumulators of their own (prefill)
   int csk;                  // > 1: launched in clusters of csk CTAs (gemm_small.cu); a
                             // row tile whose contributors share a cluster is summed by
                             // its first contributor from partials the others push into

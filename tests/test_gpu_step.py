@@ -254,3 +254,41 @@ def test_attention_of_many_vectors(H, Hkv, hd, K, lens):
             assert np.abs(z[b] - ref).max() <= 1e-3 * np.abs(ref).max()
     finally:
         eng.close()
+
+
+@pytest.mark.parametrize("rows", [144, 256])
+def test_prefill_is_as_exact_in_large_passes(rows):
+    """Values that one prefill pass of 144 or 256 rows leaves in the cache, against the
+    64-bit ones rounded to bf16: the share that differs is proportional to the error of
+    the projection's sums before they are rounded, and no larger than a pass of 128
+    rows leaves (1.5 times: about 90 of 131072 values differ there, so chance is 1.1 to
+    1.3; sums of both planes in one accumulator give 2).  Stream-K ranges of 16.8 k
+    tiles of 64: most CTA pairs work on two row tiles."""
+    from paper_2608_10362_gb300 import Engine
+    from seeded_inputs import ModelShape
+    t = ModelShape(1, 4096, 24, 8, 128, 256, 1000)
+    g = torch.Generator(device="cuda").manual_seed(31)
+    normal = lambda *shape: torch.randn(shape, device="cuda", generator=g)
+    d, f, q, kv = t.d_model, t.d_ffn, t.q_dim, t.kv_dim
+    w = {"tok_emb": normal(t.vocab, d) * 0.02, "attn_norm": 1 + 0.1 * normal(d), "wq": normal(q, d) * 0.02,
+         "wk": normal(kv, d) * 0.02, "wv": normal(kv, d) * 0.02, "wo": normal(d, q) * 0.02,
+         "ffn_norm": 1 + 0.1 * normal(d), "w_gate": normal(f, d) * 0.02, "w_up": normal(f, d) * 0.02,
+         "w_down": normal(d, f) * 0.02, "final_norm": 1 + 0.1 * normal(d), "lm_head": normal(t.vocab, d) * 0.02}
+    w = {name: v.to(torch.bfloat16) for name, v in w.items()}
+    model = ("tok_emb", "final_norm", "lm_head")
+    eng = Engine(t, [(name, -1 if name in model else 0, v) for name, v in w.items()], max_batch=1, max_seq=300,
+                 max_k=4, max_drafts=0, use_graphs=False)
+    try:
+        def share(n):
+            prompt = gen_prompt(n, n + 1, t.vocab)     # the last token is the next pass's
+            eng.prefill(0, prompt, seed=1)
+            assert eng.sync() == 0
+            got = eng.kv.view(torch.bfloat16).view(2, t.n_kv_heads, 300, t.head_dim)[1, :, :n].transpose(0, 1)
+            h = w["tok_emb"][torch.as_tensor(prompt[:n].astype(np.int64), device="cuda")].double()
+            x = h * torch.rsqrt((h * h).mean(-1, keepdim=True) + t.norm_eps) * w["attn_norm"].double()
+            ref = (x @ w["wv"].double().T).view(n, t.n_kv_heads, t.head_dim)
+            assert (got.double() - ref).abs().max() <= 2.0 ** -8 * ref.abs().max()
+            return (got != ref.to(torch.bfloat16)).double().mean().item()
+        assert 0 < share(rows) <= 1.5 * share(128)
+    finally:
+        eng.close()
