@@ -89,7 +89,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  pdl_launch_dependents();
   const uint32_t tmem_base = ctl.tmem_base;
   // optional trace (16 slots per CTA): 0 entry, 13 dependency released,
   // 2 activation loads issued, 3 first MMA, 4..11 epilogue, 1 exit
@@ -119,6 +118,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
         tma_load_2d(smem_b + static_cast<size_t>(slot) * b_bytes, &a.map_b, k_tile * kTileK, 0, &ctl.full[slot], pol_b);
       };
       pdl_wait();
+      pdl_launch_dependents();   // after the wait: see ptx.cuh
       trace_at(trace, 2);
       // the first n_pre tiles (the ring is empty: no wait needed)
       for (int p = 0; p < n_pre; ++p) {

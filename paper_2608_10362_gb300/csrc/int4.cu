@@ -56,7 +56,9 @@
 // the partial sums of a tile shared by several warps are added in warp order at the end.
 // Every sum has a fixed order: results are bit-reproducible.  Launched with
 // programmatic stream serialisation: a CTA starts its weight copies, then
-// waits for the previous kernel (whose output may be x).
+// waits for the previous kernel (whose output may be x).  The packed weights' writer is
+// complete by then: every kernel that lets the next one start early does so after its
+// own wait, and int4_pack_kernel (fence at its end) does not.
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -411,6 +413,8 @@ __global__ void int4_pack_kernel(const uint8_t* __restrict__ qweight, const bf16
     d[2] = make_uint4(zw[0] | (static_cast<uint32_t>(zw[1]) << 16), zw[2] | (static_cast<uint32_t>(zw[3]) << 16),
                       zw[4] | (static_cast<uint32_t>(zw[5]) << 16), zw[6] | (static_cast<uint32_t>(zw[7]) << 16));
   }
+  // a layer launched next may read the records before its griddepcontrol.wait
+  __threadfence();
 }
 
 }  // namespace

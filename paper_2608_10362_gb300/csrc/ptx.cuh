@@ -143,8 +143,8 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 
 // ---------------------------------------------------------------- PDL
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the next launch start once every CTA of this one has called it.  The kernels of
-// a pass call it after griddepcontrol.wait: called at the start, the next launch's
+// Lets the next launch start once every CTA of this one has called it.  Every kernel
+// calls it after griddepcontrol.wait, or not at all: called at the start, the next launch's
 // CTAs were handed out while an earlier kernel still held part of the chip, and some
 // of them started 6 us late although SMs were free by then (verify pass of the 1.1B
 // target 0.866 -> 0.821 ms, 7B 2.755 -> 2.715, batched 8B 7.25 -> 7.12).  One launch's

@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(kSThreads, NV > 2 ? 2 : 3) sample_kernel(const
 // grid (2K+1 rows, groups): row statistics per CTA; the last CTA of a group decides
 __global__ void __launch_bounds__(kSThreads) accept_kernel(const __grid_constant__ AcceptArgs a) {
   __shared__ SampleSmem sm;
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   accept_row<kSThreads>(a, blockIdx.x, blockIdx.y, sm, threadIdx.x, [] { __syncthreads(); });
 }
 

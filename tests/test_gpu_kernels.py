@@ -152,6 +152,49 @@ def test_pack_matrix_matches_documented_layout(n, k, pair):
     assert np.array_equal(got, ref)
 
 
+def test_calls_back_to_back_see_their_predecessors_output():
+    """op_linear over rows of every kernel, each reading weights and activations that
+    the work before it writes, its output drawn from by op_sample, and INT4 layers right
+    after their packing: nothing waits on the host, one scratch.  The launches may start
+    before their predecessors end; the outputs have to be those of the final inputs."""
+    from paper_2608_10362_gb300 import int4_pack, op_linear, op_linear_int4, op_sample
+    V, k, rounds = 5000, 3000, 3
+    g = torch.Generator(device="cuda").manual_seed(12)
+    normal = lambda *s: torch.randn(s, device="cuda", generator=g)
+    all_rows = (5, 16, 17, 144, 160, 161, 256)
+    ws = [(normal(V, k) * 0.02).to(torch.bfloat16) for _ in range(2)]
+    xs = {r: [normal(r, k).to(torch.bfloat16) for _ in range(2)] for r in all_rows}
+    u = {r: torch.rand(r, device="cuda", generator=g).clamp(1e-6, 1 - 1e-6) for r in all_rows}
+    codes = [torch.randint(0, 256, (V, 2048 // 2), dtype=torch.uint8, device="cuda", generator=g) for _ in range(2)]
+    scales = torch.full((V, 16), 0.005, dtype=torch.bfloat16, device="cuda")
+    zeros = torch.full((V, 16), 8, dtype=torch.uint8, device="cuda")
+    x4 = normal(5, 2048).to(torch.bfloat16)
+    w = torch.empty_like(ws[0])
+    x = {r: torch.empty_like(xs[r][0]) for r in all_rows}
+    scratch = torch.zeros(64 << 20, dtype=torch.uint8, device="cuda")
+    got = []
+    for i in range(rounds):
+        for r in all_rows:
+            torch.add(ws[i % 2], 0, out=w)
+            torch.add(xs[r][i % 2], 0, out=x[r])
+            y = op_linear(x[r], w, scratch)
+            t = op_sample(y, 0.9, u[r])
+            got.append((r, i % 2, y, t, op_sample(y, 0.0)))
+        y4 = op_linear_int4(x4, int4_pack(codes[i % 2], scales, zeros), V)
+        got.append((0, i % 2, y4, op_sample(y4, 0.9, u[5]), op_sample(y4, 0.0)))
+    torch.cuda.synchronize()
+    for r, i, y, t, greedy in got:
+        if r:
+            a, b = xs[r][i].double(), ws[i].double()
+            bound = 1e-4 * (a.abs() @ b.abs().T) + 1e-6
+        else:   # sums of 128 terms x (128 + q), the zero point's (128 + 8) x beside them
+            a, s = x4.double(), scales[0, 0].double()
+            b = (torch.stack([codes[i] & 15, codes[i] >> 4], -1).view(V, -1).double() - 8) * s
+            bound = 2.0 ** -24 * (128 * (256 + 15 + 8) * s * a.abs().sum(1, keepdim=True) + 8 * (a.abs() @ b.abs().T))
+        assert ((y.double() - a @ b.T).abs() <= bound).all(), (r, i)
+        assert torch.equal(greedy, y.argmax(1).int()) and torch.equal(t, op_sample(y, 0.9, u[r or 5])), (r, i)
+
+
 @pytest.mark.parametrize("T", [0.0, 1.0, 0.8])
 @pytest.mark.parametrize("vocab", [2048, 32000, 128256, 97])
 def test_sampler_matches_inverse_cdf(T, vocab):
