@@ -183,8 +183,8 @@ def test_tiny_prompt_edge_cases(tiny):
 def test_verify_pass_row_counts(B, K):
     """One verify pass at 2, 8, 9, 12, 18, 33, 128, 135, 160 and 256 rows (up to 8: the
     small GEMM; above: the CTA-pair GEMM's operand layouts, two planes side by side up
-    to 128 rows, one after the other above), requests of different lengths: every request's logits and new K/V against
-    the oracle at the step tests' tolerance."""
+    to 128 rows, one after the other above), requests of different lengths: every
+    request's logits, keys and values against the oracle at the step tests' tolerance."""
     from oracle.llama import LlamaOracle
     from paper_2608_10362_gb300 import Engine, _lib
     from seeded_inputs import SHAPES, gen_prompt, gen_weights
@@ -209,10 +209,11 @@ def test_verify_pass_row_counts(B, K):
             ref = oracle.forward(cache, rows)[-(K + 1):]
             assert np.abs(z[b] - ref).max() <= 1e-3 * np.abs(ref).max()
             n = len(rows)
-            k_ref = np.stack([np.asarray(cache.k[l])[:n] for l in range(t.n_layers)])   # [layer][pos][head][hd]
-            got = kv[:, 0, b, :, :n].transpose(0, 2, 1, 3)
-            # bf16 values: at most one rounding step apart
-            assert np.abs(got - k_ref).max() <= 2.0 ** -7 * np.abs(k_ref).max()
+            for side, cached in enumerate((cache.k, cache.v)):   # [layer][pos][head][hd]
+                kv_ref = np.stack([np.asarray(cached[l])[:n] for l in range(t.n_layers)])
+                got = kv[:, side, b, :, :n].transpose(0, 2, 1, 3)
+                # bf16 values: at most one rounding step apart
+                assert np.abs(got - kv_ref).max() <= 2.0 ** -7 * np.abs(kv_ref).max()
     finally:
         eng.close()
 
