@@ -844,7 +844,6 @@ void small_gemm(GemmArgs& a, int* grid) {
   const int planes = a.split ? 2 : 1;
   const CskPick pk = pick_csk(a, planes, gemm_grid(a.row_tiles, a.k_tiles));
   *grid = pk.grid;
-  a.small = 1;
   a.csk = pk.csk;
   a.n_pad = 16;
   a.stages = gemm_small_stages(planes, a.csk);
@@ -852,7 +851,6 @@ void small_gemm(GemmArgs& a, int* grid) {
 
 // `pass`: an op of the persistent pass kernel.
 memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, bool pass, std::vector<PassOp>& ops) {
-  const int planes = a.split ? 2 : 1;
   a.partials = c->gemm_part;
   a.counters = c->gemm_cnt;
   a.status = c->status;
@@ -875,13 +873,10 @@ memspec_status emit_gemm(memspec_ctx* c, GemmArgs& a, bool pass, std::vector<Pas
   }
   PassOp op{};
   op.type = OP_GEMM;
-  op.grid = gemm_grid(a.row_tiles, a.k_tiles);
-  if (pass) {   // the persistent kernel runs every op on its own grid
-    a.stages = gemm_pick_stages(a.n_pad, planes);
-    op.smem = static_cast<int>(gemm_smem_bytes(a.n_pad, a.stages, planes));
-  } else {
+  if (pass)
+    op.grid = gemm_grid(a.row_tiles, a.k_tiles);
+  else
     small_gemm(a, &op.grid);
-  }
   op.u.g = a;
   ops.push_back(op);
   return MEMSPEC_OK;

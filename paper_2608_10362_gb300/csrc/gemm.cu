@@ -268,8 +268,8 @@ static int gemm_budget_bytes() {
   return 200 * 1024;
 }
 
-int gemm_pick_stages(int n_pad, int planes) {
-  const int stage = kABytes + n_pad * 128 * planes;
+int gemm_pick_stages(int n_pad) {
+  const int stage = kABytes + n_pad * 128;
   const int budget = gemm_budget_bytes();
   const int fixed = kTileM * kStagePitch * 4 + kMaxRows * 4 + static_cast<int>(sizeof(EpiCtx)) + 1024;
   int s = (budget - fixed) / stage;
@@ -278,8 +278,8 @@ int gemm_pick_stages(int n_pad, int planes) {
   return s;
 }
 
-size_t gemm_smem_bytes(int n_pad, int stages, int planes) {
-  return static_cast<size_t>(stages) * (kABytes + n_pad * 128 * planes) + kTileM * kStagePitch * 4 +
+size_t gemm_smem_bytes(int n_pad, int stages) {
+  return static_cast<size_t>(stages) * (kABytes + n_pad * 128) + kTileM * kStagePitch * 4 +
          kMaxRows * 4 + sizeof(EpiCtx) + 1024;
 }
 

@@ -144,10 +144,9 @@ struct GemmArgs {
   int split_epi;            // 1: contributors to a split row tile only store their partials;
                             // gemm_split_epi_kernel (the next launch) sums them and runs the
                             // epilogue, one CTA per (row tile, 16-row chunk)
-  int small;                // 1: gemm_small.cu's kernel (n_pad 16); x4d: 1: map_b, map_b2
-  int x4d;                  // are 4-D maps of the activations {64 columns, rows, planes, k tiles}
-                            // with boxes of one and of gemm_small_x_group k tiles; 0: 2-D maps
-                            // of the planes
+  int x4d;                  // gemm_small.cu (n_pad 16), 1: map_b, map_b2 are 4-D maps of the
+                            // activations {64 columns, rows, planes, k tiles} with boxes of
+                            // one and of gemm_small_x_group k tiles; 0: 2-D maps of the planes
   int w_after_wait;         // gemm_small.cu, gemm_pair.cu, 1: the weights too are read only after
                             // griddepcontrol.wait (an op-level call's weights may be anything
                             // that earlier work on the stream writes)
@@ -349,8 +348,8 @@ cudaError_t launch_int4_pack(const uint8_t* qweight, const bf16* scales, const u
 // launchers (each returns the launch's cudaError_t)
 cudaError_t launch_embed(const EmbedArgs& a, int rows, cudaStream_t s, bool pdl);
 cudaError_t launch_gemm(const GemmArgs& a, int grid, size_t smem, cudaStream_t s, bool pdl);
-size_t gemm_smem_bytes(int n_pad, int stages, int planes = 1);
-int gemm_pick_stages(int n_pad, int planes = 1);
+size_t gemm_smem_bytes(int n_pad, int stages);
+int gemm_pick_stages(int n_pad);
 cudaError_t gemm_set_max_smem();
 cudaError_t launch_gemm_split_epi(const GemmArgs& a, int gemm_grid, cudaStream_t s, bool pdl);
 // gemm_small.cu: ring stages, shared memory, thread-block clusters of csk CTAs that

@@ -14,8 +14,7 @@ struct alignas(64) PassOp {
   int type;
   int grid;       // OP_GEMM: stream-K grid (CTAs with tiles)
   int n_units;    // OP_EMBED rows, OP_ATTN units, OP_SAMPLE groups, OP_ACCEPT rows x groups
-  int smem;       // OP_GEMM as its own launch: dynamic shared memory bytes
-  int pad[12];
+  int pad[13];
   union U {
     GemmArgs g;
     AttnArgs at;
