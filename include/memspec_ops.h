@@ -21,11 +21,13 @@ memspec_status memspec_op_linear_scratch_bytes(int32_t rows, int32_t n_out, int3
                                                size_t* bytes);
 
 /* y[rows][n_out] (fp32) = x[rows][k] (bf16, row-major) . w[n_out][k]^T (bf16).
- * This is the weight-streaming GEMM every projection of the verify and draft
- * passes runs (Q/K/V, O, gate/up, down, LM head): TMA-staged weight tiles,
- * tcgen05 MMA into TMEM, stream-K over all SMs, deterministic split-K
- * reduction (above 16 rows, split row tiles are finished by a second launch
- * on the same stream, one CTA per row tile and 16-row chunk).
+ * A weight-streaming GEMM: TMA-staged weight tiles, tcgen05 MMA into TMEM,
+ * stream-K over the SMs, deterministic split-K reduction (above 16 rows, split
+ * row tiles are finished by a second launch on the same stream, one CTA per
+ * row tile and 16-row chunk).  Up to 16 rows and from 161 it runs the kernels
+ * of the verify and draft passes' projections (Q/K/V, O, gate/up, down, LM
+ * head) with one activation plane for their two; from 17 to 160 one that no
+ * pass runs.
  * rows in 1..256, k a multiple of 8, n_out >= 1, and
  * ceil(n_out/128) * ceil(k/64) * (SMs + 1) below 2^32.
  * scratch_dev: memspec_op_linear_scratch_bytes bytes, 256-byte aligned, zeroed
@@ -39,20 +41,20 @@ memspec_status memspec_op_linear(const void* x_dev, const void* w_dev, float* y_
                                  void* scratch_dev, size_t scratch_bytes,
                                  uint32_t* status_dev, void* stream);
 
-/* The same GEMM as memspec_op_linear (y = x . w^T, fp32 out), for callers
- * that cannot allocate device memory: plug-ins whose host application owns all
- * device memory, fixed-budget deployments that allocate only at start-up, and
- * latency-critical loops that cannot afford cudaMalloc / cudaFree (which may
- * synchronise the device).  The paper has no counterpart; this is a property
- * of the library's interface.
+/* The same product as memspec_op_linear (y = x . w^T, fp32 out), by the kernel
+ * that it runs for 17 to 160 rows, for callers that cannot allocate device
+ * memory: plug-ins whose host application owns all device memory, fixed-budget
+ * deployments that allocate only at start-up, and latency-critical loops that
+ * cannot afford cudaMalloc / cudaFree (which may synchronise the device).  The
+ * paper has no counterpart; this is a property of the library's interface.
  * Instead of a scratch argument it uses one file-scope device array of about
  * 2.6 MB that every GPU loading the library keeps until the process exits.
  * Limits: rows in 1..16, n_out in 1..131072, k a positive multiple of 8 up to
  * 2^20; x and w 16-byte aligned.  Larger sizes return MEMSPEC_ERR_INVALID_ARG
  * (message in memspec_op_last_error) and enqueue nothing.  The call allocates
  * nothing; it enqueues a clear of the array's counters and the kernel on
- * `stream`.  Its split-K grid differs from memspec_op_linear's, so results
- * agree with it within rounding, not bit for bit.
+ * `stream`.  Its kernel and split-K grid differ from memspec_op_linear's, so
+ * results agree with it within rounding, not bit for bit.
  * All calls share the array: calls that overlap on the GPU (other streams,
  * other host threads) race - serialise them.  The first call on a device looks
  * up the array's address on that device; make it before any stream capture.

@@ -750,8 +750,9 @@ struct FwdSpec {
 // bandwidth on small matrices).  kGemmSpareSms SMs stay free: with every SM
 // streaming, some SMs stream 1-2 us slower than the rest and the CTAs that start
 // on SMs still held by the previous launch start late, and a static partition
-// waits for the slowest; with 16 SMs free the verify pass measured 3.34 ms
-// instead of 3.42 (QKV launch 21 us instead of 25).
+// waits for the slowest.  7B verify pass at 2048 keys (gemm_small.cu), ms with so many SMs
+// free: 0 2.750, 4 2.761, 8 2.698, 16 2.683, 24 2.681, 40 2.809; the 1.1B's at 512 keys
+// 0.823, 0.822, 0.823, 0.825, 0.832, 0.855; the 160M's of two rows 0.290 with any.
 constexpr int kGemmSpareSms = 16;
 
 int env_int(const char* name, int dflt) {
@@ -829,10 +830,20 @@ CskPick pick_csk(const GemmArgs& a, int planes, int g0) {
 
 // CTA pairs of gemm_pair.cu for `rows` activation rows, 0: gemm.cu's kernel.  One
 // pair per two SMs, and ranges of at least a quarter of a row-tile pair.
-// Two planes: from 9 rows (gemm_small.cu takes up to 8).  Verify pass of 6 layers of the 8B target, this kernel /
-// gemm.cu's: 18 rows 0.784 / 0.836 ms, 54 rows 0.911 / 1.060, 144 rows 1.292 / 1.559.
-// One plane (memspec_op_linear): from 161 rows.  28672 x 4096 at 144 rows 57.1 / 58.2
-// us but 12288 x 4096 27.2 / 25.9; at 256 rows 71.5 / 85.6 and 32.3 / 35.0.
+// Two planes: from 9 rows (gemm_small.cu takes up to 8).  Verify pass of 6 layers of the
+// 8B target, this kernel / gemm.cu's with every other kernel the same: 18 rows 0.784 /
+// 0.836 ms, 54 rows 0.911 / 1.060, 144 rows 1.292 / 1.559.  At 9 to 16 rows only whole
+// passes were compared, now / with all the kernels before gemm_small.cu, gemm_pair.cu and
+// attn_tc.cu: 8 layers of the 7B 0.771 to 0.779 / 0.890 to 0.934 ms, the 1.1B 1.03 to
+// 1.04 / 1.70 to 1.80, the 160M 0.414 to 0.421 / 0.609 to 0.651.
+// One plane (memspec_op_linear): from 161 rows, where most sizes gain.  us, this kernel /
+// gemm.cu's (n_out x k):
+//   rows    28672 x 4096   4096 x 11008   12288 x 4096   4096 x 4096   2304 x 768
+//   144     55.0 / 55.5    22.2 / 22.0    25.5 / 23.7    13.6 / 13.3   8.1 / 7.7
+//   145-160 56.9 / 60.9    22.3 / 23.5    26.0 / 25.4    13.8 / 13.8   8.2 / 7.9
+//   161     58.6 / 63.6    22.3 / 23.9    26.8 / 26.0    13.8 / 14.1   8.5 / 8.0
+//   193     63.1 / 68.6    24.3 / 24.8    28.5 / 28.2    15.7 / 14.9   8.9 / 8.4
+//   256     69.6 / 81.2    24.1 / 27.4    30.5 / 32.7    15.4 / 16.2   9.4 / 9.0
 int gemm_pairs(int rows, int split, int row_tiles, int k_tiles) {
   if (rows < (split ? 9 : 161)) return 0;
   const int T = (row_tiles + 1) / 2 * k_tiles;

@@ -15,7 +15,8 @@
 // 128, 300 to 3000 keys.)  A thread owns an MMA
 // row, so the softmax has no cross-lane step; its running max only follows a tile's
 // when that is more than 2^8 larger (exact: every use of it cancels), which leaves
-// rescaling O to a few tiles.  Units of fewer vectors repeat them: with kKG = 64 (32)
+// rescaling O to a few tiles (as published for FlashAttention-4; two softmax groups
+// that alternate, below: FlashAttention-3).  Units of fewer vectors repeat them: with kKG = 64 (32)
 // keys per thread the 128 rows are 2 (4) copies of up to 64 (32) vectors, copy j takes
 // keys [j kKG, (j + 1) kKG) of each tile and has zeros for the others in P.
 // Two softmax warpgroups take the even and the odd tiles, each with its own S, O, max

@@ -47,7 +47,8 @@
 // per record (small copies: per-request cost decides, and 1 KB bulk copies
 // were slower).  Rings of 3, 4 and 6 slots are no faster (GB300, 12288 x 4096 at 5 rows:
 // 8.9 us with 2, 9.2 with 3 or 4): a record costs an SM 62 cycles where HBM would allow
-// 46.  Tried instead: two CTAs per SM, 9.5 us; a warp per column range with its
+// 46, and whole tiles leave SMs without work (768 tiles are 6 on each of 128 CTAs, 256 are
+// 2 on each of 128; 152 SMs).  Tried instead: two CTAs per SM, 9.5 us; a warp per column range with its
 // activations in registers and the records loaded straight to registers, 9.8 (8.7 of it
 // with every record in L2: unpacking and MMAs, ALU pipe 48% and issue 46% busy).  The
 // activations arrive as one 1-D bulk copy (TMA) per row, outside the load/store unit's
